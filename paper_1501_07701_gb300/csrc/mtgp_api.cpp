@@ -376,7 +376,7 @@ mtgp_status mtgp::build_work(uint32_t n_streams, const uint32_t* ids, const uint
 size_t mtgp::table_bytes(const Work& w, size_t* items_off, size_t* segs_off)
 {
     const size_t a = 256;
-    const size_t io = a;
+    const size_t io = kCounterBytes;
     const size_t so = io + ((w.items.size() * sizeof(WorkItem) + a - 1) / a) * a;
     if (items_off)
         *items_off = io;
@@ -389,7 +389,7 @@ void mtgp::fill_table(const Work& w, void* host)
 {
     size_t io, so;
     table_bytes(w, &io, &so);
-    std::memset(host, 0, io);   // work counter (first word) = 0
+    std::memset(host, 0, io);   // claim counters
     if (!w.items.empty())
         std::memcpy((char*)host + io, w.items.data(), w.items.size() * sizeof(WorkItem));
     if (!w.segs.empty())
@@ -566,6 +566,10 @@ extern "C" mtgp_status mtgp_init_statuses(mtgp_params_t params, const uint32_t* 
         return fail_cuda(e, "cudaGetDevice");
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
+    if ((e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device)) != cudaSuccess) {
+        delete h;
+        return fail_cuda(e, "SM count");
+    }
     auto bail = [&](cudaError_t err, const char* what) {
         mtgp_status st = fail_cuda(err, what);
         destroy_streams(h);
@@ -677,17 +681,50 @@ extern "C" mtgp_status mtgp_init_statuses_multi(const mtgp_params_t* sets, uint3
 
 LaunchCfg mtgp::default_config(const KParams& P)
 {
-    // 8 warps per SM; 128-word software-pipelined steps when the parameter
+    // 8 warps per SM, in one CTA; 128-word software-pipelined steps when the parameter
     // set allows them (N - pos >= 256), else 256-word steps, else 128, else
     // 64 (short states such as Mexp 3217).
     LaunchCfg c;
-    c.warps_per_cta = 4;
-    c.ctas_per_sm = 2;
+    c.warps_per_cta = 8;
+    c.ctas_per_sm = 1;
     c.k = 4;
     c.kernel = 0;
     c.coop_percent = 0;
     if (P.n - P.pos < 256u || !fast_supported(P, 4))
         c.k = fast_supported(P, 8) ? 8 : (fast_supported(P, 4) || !fast_supported(P, 2) ? 4 : 2);
+    c.automatic = fast_supported(P, c.k, 8) && fast_supported(P, c.k, 4);
+    if (!c.automatic) {   // the ring kernel: large states leave room for four warps per CTA
+        c.warps_per_cta = 4;
+        c.ctas_per_sm = 2;
+    }
+    return c;
+}
+
+LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
+                           uint64_t max_item)
+{
+    LaunchCfg c = cfg;
+    if (!cfg.automatic || n_items == 0)
+        return c;
+    c.warps_per_cta = 8;
+    c.ctas_per_sm = 1;
+    const uint64_t sms = (uint64_t)st->sms;
+    if (n_items <= 4u * sms) {
+        // one warp per SM quarter: a second one on the same quarter slows
+        // both (456 streams of 2^20, Mexp 11213: 0.93 ms on 8-warp CTAs
+        // whose three busy warps may share a quarter, 0.53 apart)
+        c.warps_per_cta = 4;
+        c.ctas_per_sm = 1;
+    } else if (total / std::max<uint64_t>(max_item, 1) >= 12u * sms ||
+               (n_items > 8u * sms && max_item * n_items <= total + total / 8u)) {
+        // 12 warps per SM run 1-2 % faster than 8 and end evenly, when no
+        // stream is longer than a warp's share of the launch at 12 (or when
+        // all are about equal): 4096 x 2^18 takes 0.79 ms at 12 and 0.89 at 8,
+        // but the uneven workload, whose longest stream is a warp's share at
+        // 8, takes 4.3 ms at 12 and 3.6 at 8
+        c.warps_per_cta = 4;
+        c.ctas_per_sm = 3;
+    }
     return c;
 }
 
@@ -750,20 +787,24 @@ extern "C" mtgp_status mtgp_get_statuses(mtgp_streams_t st, uint32_t* states, vo
 mtgp_status mtgp::geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, Geometry* g)
 {
     const auto key = std::make_tuple(cfg.warps_per_cta, cfg.ctas_per_sm, cfg.k, cfg.kernel);
-    if (!(st->geo_valid && st->geo_key == key)) {
+    auto it = st->geo_caps.find(key);
+    if (it == st->geo_caps.end()) {
         Geometry full;
         cudaError_t e = plan_geometry(st->P.k, cfg, 0x7FFFFFFF, st->device, &full);
         if (e != cudaSuccess)
             return fail_cuda(e, "launch geometry");
-        st->geo_cap = full;
-        st->geo_key = key;
-        st->geo_valid = true;
+        it = st->geo_caps.emplace(key, full).first;
     }
-    *g = st->geo_cap;
-    // One CTA per item at most (a CTA may take a whole stream); CTAs that find
-    // no work left exit at once.
-    const long long want = (long long)n_items;
-    g->grid = (int)std::max(1LL, std::min<long long>(want, st->geo_cap.grid));
+    *g = it->second;
+    // One CTA per item at most (a CTA may take a whole stream), and without
+    // CTA-wide streams no more CTAs per SM than give every item a warp.
+    const long long items = (long long)n_items;
+    long long want = items;
+    if (cfg.coop_percent == 0 && g->kernel == 0) {
+        const long long slots = (long long)st->sms * (g->threads / 32);
+        want = std::min<long long>(want, st->sms * ((items + slots - 1) / slots));
+    }
+    g->grid = (int)std::max(1LL, std::min<long long>(want, it->second.grid));
     return MTGP_OK;
 }
 
@@ -823,7 +864,8 @@ mtgp_status mtgp::launch_work_table(mtgp_streams* st, const Work& w, void* table
     size_t io, so;
     table_bytes(w, &io, &so);
     Geometry g;
-    mtgp_status stt = geometry_for(st, cfg, (uint32_t)w.items.size(), &g);
+    const LaunchCfg run = fit_config(st, cfg, (uint32_t)w.items.size(), w.total, w.max_item);
+    mtgp_status stt = geometry_for(st, run, (uint32_t)w.items.size(), &g);
     if (stt != MTGP_OK)
         return stt;
     GenArgs a;
@@ -1078,6 +1120,7 @@ mtgp_status mtgp::validate_config(const mtgp_launch_config* c, LaunchCfg* out)
     out->k = (int)c->words_per_lane;
     out->kernel = (int)c->kernel;
     out->coop_percent = (int)c->coop_percent;
+    out->automatic = false;
     return MTGP_OK;
 }
 
@@ -1111,6 +1154,7 @@ std::vector<LaunchCfg> mtgp::tuning_candidates(const KParams& P)
         x.k = k;
         x.kernel = 0;
         x.coop_percent = coop;
+        x.automatic = false;
         v.push_back(x);
     };
     for (int k : {8, 4, 2}) {
@@ -1136,6 +1180,7 @@ std::vector<LaunchCfg> mtgp::tuning_candidates(const KParams& P)
             x.k = 8;
             x.kernel = 1;
             x.coop_percent = 0;
+            x.automatic = false;
             v.push_back(x);
         }
     }
@@ -1296,8 +1341,6 @@ static mtgp_status record_graph(mtgp_plan* p)
     if (e1 == cudaSuccess)
         e1 = launch_jump_batch(p->st, p->d_rows, p->d_jitems, n_jumps, p->d_jpolys, p->jumps.words,
                                p->jumps.smem, cap);
-    if (e1 == cudaSuccess)
-        e1 = cudaMemsetAsync(p->d_table, 0, 2 * sizeof(uint32_t), cap);
     GenArgs a;
     a.P = p->st->P.k;
     a.states = split ? p->d_rows : p->st->d_states;
@@ -1313,6 +1356,10 @@ static mtgp_status record_graph(mtgp_plan* p)
     a.trace = p->d_trace;
     a.sets = p->st->d_sets;
     a.set_of = split ? p->d_row_set : p->st->d_set_of;
+    const bool counted = p->stats || p->geo.kernel != 0 || a.n_coop ||
+                         !items_placed(p->n_items, (uint32_t)p->geo.grid, (uint32_t)p->geo.threads / 32u);
+    if (e1 == cudaSuccess && counted)
+        e1 = cudaMemsetAsync(p->d_table, 0, kCounterBytes, cap);
     cudaError_t e2 = e1;
     if (e2 == cudaSuccess && p->stats) {
         // the fused kernel writes every request's counts; requests with no
@@ -1440,6 +1487,7 @@ static mtgp_status build_launch(mtgp_plan* p, uint64_t max_piece)
         CUDA_TRY(cudaMalloc(&p->d_trace, (size_t)p->n_items * 4 * sizeof(uint64_t)), "cudaMalloc(trace)");
         CUDA_TRY(cudaMemset(p->d_trace, 0, (size_t)p->n_items * 4 * sizeof(uint64_t)), "cudaMemset");
     }
+    p->cfg = fit_config(st, p->cfg, p->n_items, p->split.work.total, p->max_item);
     return geometry_for(st, p->cfg, p->n_items, &p->geo);
 }
 

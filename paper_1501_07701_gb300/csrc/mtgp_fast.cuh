@@ -236,68 +236,154 @@ __device__ __forceinline__ void gen_row(uint32_t (&r)[(M + WG - 1) / WG], uint32
 
 // ===========================================================================
 // nfull consecutive full rows of one request, single warp, software-pipelined
-// steps of W = 128 words (K = 4 sub-steps).
+// steps of W = 128 words (K = 4 sub-steps), with the tempering one row late.
+//
+// Late tempering.  The word i+pos that the recursion of number i picks up is
+// the tempering word of number i+1, whose state word x_{i+1+N} is what the
+// same lane reads as its neighbour word one row later.  So a lane looks up
+// the tempering of number i+1 when it picks the word up, keeps it in T[m] for
+// a row, and stores number i+1 when it reads x_{i+1+N}: one shared load less
+// per number than reading word i+pos-1 again.  Row q of the run thus stores
+// the numbers (q-1)N+1 .. qN; the last row's remaining numbers are stored
+// after the loop.  Number 0 of the run is the one that column N-1 stores in
+// the first row, from a T set up before it.
+//
+// Qp[m] is this lane's pick-up address for column group m, with the wrap at
+// column N in it: a wrapped pick-up reads the new row's word at its own place
+// in S, so nothing is mirrored behind the row.
 //
 // When N - pos >= 2W, the loads of step s+1 never touch a word that step s
 // writes: word i+1 and the unwrapped pick-ups lie beyond step s's columns,
-// and a wrapped pick-up (mirror) of a column c < W(s+2) lands below
-// c + pos - N < Ws.  The same holds from the last step of a row to the first
-// step of the next (its pick-ups end below pos + W <= N - W, where the last
-// step begins at or above N - W).  So the loads of step s+1 are issued
-// before the stores of step s, and one __syncwarp per step (after the
-// stores) orders every store before the loads that read it two steps later.
-// The loads issued during a row's last step are those of step 0 (the same
-// addresses in every row); after the last row they are simply unused.
+// and a wrapped pick-up of a column c < W(s+2) lands below c + pos - N < Ws.
+// The same holds from the last step of a row to the first step of the next
+// (its pick-ups end below pos + W <= N - W, where the last step begins at or
+// above N - W).  So the loads of step s+1 are issued before the stores of
+// step s, and one __syncwarp per step (after the stores) orders every store
+// before the loads that read it two steps later.  The neighbour of column
+// N-1 is column 0 of the new row (`x1_last` points there): written in step 0
+// and read in step NS-2 >= 1 or later.  The loads issued during a row's last
+// step are those of step 0 (the same addresses in every row); after the last
+// row they are simply unused.  Lanes past column N-1 in the last group
+// compute on the words behind the row and write there; only their output
+// store is predicated off.
+//
+// What bounds it (ncu, 1216 streams, 8 warps per SM, Mexp 11213): 6.03 LSU and
+// 11.4 ALU instructions per 32 numbers, LSU data stage 85 % and ALU 74 % busy
+// (the loop it replaced: 7.34 and 13.3).  Hence the late tempering and the
+// wrapped addresses (LSU), the packed folds and the multiply for the left
+// shift (ALU).  The rows are unrolled because a row of three steps leaves its
+// pointer and register moves exposed: one stream alone took 0.62 ms for 2^20
+// numbers with one row per pass, 0.51 with four.  All together: the uneven
+// workload 4.72 -> 3.61 ms (1085 -> 1419 Gnumbers/s, 0.84 of the HBM rate),
+// 4096 x 2^18 at 12 warps per SM 1.02 -> 0.79 ms, one stream of 2^20 numbers
+// 0.75 -> 0.51 ms; Mexp 44497, 1024 x 2^20, 1.15 -> 0.95 ms.
 // ===========================================================================
+__device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t lds(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+// Table addresses (less the table's offset) of four tempering words at once:
+// their 16-bit and 8-bit folds run packed, two and four words to a register,
+// and one byte permute per word then puts 4 * index under the table base tb,
+// a multiple of 256.  13 ALU instructions for four words, 16 one by one.
+__device__ __forceinline__ void temper_addr(const uint32_t (&x)[4], uint32_t tb, uint32_t (&a)[4])
+{
+    const uint32_t u = __byte_perm(x[0], x[1], 0x5410) ^ __byte_perm(x[0], x[1], 0x7632);
+    const uint32_t v = __byte_perm(x[2], x[3], 0x5410) ^ __byte_perm(x[2], x[3], 0x7632);
+    const uint32_t w = ((__byte_perm(u, v, 0x6420) ^ __byte_perm(u, v, 0x7531)) & 0x0F0F0F0Fu) * 4u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        a[i] = __byte_perm(w, tb, 0x7650 + i);
+}
+
+template <int FMT>
+__device__ __forceinline__ uint32_t finish(uint32_t v, uint32_t t)
+{
+    if (FMT == 0)
+        return v ^ t;
+    const uint32_t b = (v >> 9) ^ t;
+    if (FMT == 1)
+        return b;
+    return __float_as_uint(__uint_as_float(b) - 1.0f);
+}
+
 template <int M, int FMT>
-__device__ __forceinline__ void gen_rows_pipelined(uint32_t (&r)[M], uint32_t* Sw, uint32_t* ow,
-                                                   const uint32_t* Q, const RowP& P, uint32_t lane,
-                                                   const uint32_t* __restrict__ Tb, uint32_t last_lane,
-                                                   uint32_t nfull)
+__device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
+                                              const uint32_t* __restrict__ Tb, uint32_t nfull)
 {
     constexpr int K = 4;
     constexpr int NS = (M + K - 1) / K;   // steps per row (>= 3 here)
-    const uint32_t N = P.n;
-    uint32_t x1[K], xp[K], xq[K];
+    constexpr int U = NS <= 3 ? 4 : 2;    // rows per pass of the unrolled loop
+    const uint32_t N = P.n, last_lane = (N - 1u) & 31u;   // lane of column N-1 (group M-1)
+    uint32_t sa = saddr(S + lane);
+    uint32_t x1_last = lane >= last_lane ? saddr(S) : sa + 128u * (M - 1) + 4u;
+    uint32_t tb = saddr(Tb);
+    // the left shift as a multiply by a power of two that the compiler cannot
+    // see through: the FMA pipe is idle, the ALU pipe is not
+    uint32_t mul1 = 1u << P.sh1;
+    asm volatile("" : "+r"(mul1), "+r"(sa), "+r"(x1_last), "+r"(tb));
+    uint32_t r[M], qa[M], T[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const uint32_t p = 32u * (uint32_t)m + lane + P.pos;
+        r[m] = lds(sa + 128u * m);
+        qa[m] = saddr(S + (p < N ? p : p - N));
+        asm volatile("" : "+r"(qa[m]));   // kept, not worked out again in the loop
+        T[m] = 0u;
+    }
+    T[M - 1] = tbl(Tb, FMT == 0 ? 16u : 32u, temper_index(S[P.pos - 1u]));
+    uint32_t x1[K], xp[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
-        x1[i] = Sw[32 * i + 1];
-        xp[i] = Q[32 * i];
-        xq[i] = Q[32 * i - 1];
+        x1[i] = lds(sa + 128u * i + 4u);
+        xp[i] = lds(qa[i]);
     }
-    for (uint32_t q = 0; q < nfull; ++q, ow += N) {
+    uint32_t* op = ow + 1 - (int)N;   // where column `lane` of this row stores
+#pragma unroll U
+    for (uint32_t q = 0; q < nfull; ++q, op += N) {
+        const bool body = q != 0u;
+        const bool last = lane == last_lane || (body && lane < last_lane);
 #pragma unroll
         for (int st = 0; st < NS; ++st) {
             const int s0 = st * K;
             const int n0 = (st + 1 < NS) ? s0 + K : 0;   // next step (next row's first)
-            uint32_t y1[K], yp[K], yq[K];
+            uint32_t y1[K], yp[K];
 #pragma unroll
             for (int i = 0; i < K; ++i) {
                 if (n0 + i < M) {
-                    y1[i] = Sw[32 * (n0 + i) + 1];
-                    yp[i] = Q[32 * (n0 + i)];
-                    yq[i] = Q[32 * (n0 + i) - 1];
+                    y1[i] = n0 + i + 1 < M ? lds(sa + 128u * (n0 + i) + 4u) : lds(x1_last);
+                    yp[i] = lds(qa[n0 + i]);
                 }
             }
+            uint32_t ta[K];
+            temper_addr(xp, tb, ta);
             uint32_t xn[K], o[K];
 #pragma unroll
             for (int i = 0; i < K; ++i) {
-                if (s0 + i < M) {
-                    const uint32_t yy = (r[s0 + i] & P.mask) ^ x1[i];
-                    const uint32_t y = yy ^ (yy << P.sh1) ^ (xp[i] >> P.sh2);
+                const int m = s0 + i;
+                if (m < M) {
+                    const uint32_t yy = (r[m] & P.mask) ^ x1[i];
+                    const uint32_t y = yy ^ (yy * mul1) ^ (xp[i] >> P.sh2);
                     xn[i] = y ^ tbl(Tb, 0u, y);
-                    o[i] = temper_convert<FMT>(xn[i], temper_index(xq[i]), Tb);
+                    o[i] = finish<FMT>(x1[i], T[m]);
+                    T[m] = lds(ta[i] + (FMT == 0 ? 64u : 128u));
                 }
             }
 #pragma unroll
             for (int i = 0; i < K; ++i) {
                 const int m = s0 + i;
-                if (m < M && (m + 1 < M || lane <= last_lane)) {
+                if (m < M) {
                     r[m] = xn[i];
-                    Sw[32 * m] = xn[i];
-                    if (32u * (uint32_t)m < P.mirror)
-                        Sw[32 * m + N] = xn[i];
-                    __stcs(ow + 32 * m, o[i]);
+                    sts(sa + 128u * m, xn[i]);
+                    if (m + 1 < M ? body : last)
+                        __stcs(op + 32 * m, o[i]);
                 }
             }
             __syncwarp();
@@ -306,11 +392,120 @@ __device__ __forceinline__ void gen_rows_pipelined(uint32_t (&r)[M], uint32_t* S
                 if (n0 + i < M) {
                     x1[i] = y1[i];
                     xp[i] = yp[i];
-                    xq[i] = yq[i];
                 }
             }
         }
     }
+    // the last row's numbers after its first
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const uint32_t v = lds(sa + 128u * m + 4u);
+        if (m + 1 < M || lane < last_lane)
+            __stcs(op + 32 * m, finish<FMT>(v, T[m]));
+    }
+}
+
+// A row on the same layout (no mirror) with its numbers stored at once:
+// columns 0 .. n_valid-1.  SLOW: the row crosses into another request and
+// every lane finds its own; otherwise the row's numbers go to `ow`.
+template <int M, int FMT, bool SLOW>
+__device__ __forceinline__ void gen_row_part(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
+                                             const uint32_t* __restrict__ Tb, uint32_t n_valid,
+                                             uint64_t row_g, const Segment* __restrict__ segs,
+                                             uint32_t s_first, uint32_t s_end, uint32_t* __restrict__ out)
+{
+    constexpr int K = 4;
+    const uint32_t N = P.n;
+    uint32_t* const Sw = S + lane;
+#pragma unroll 1
+    for (uint32_t c0 = 0; c0 < n_valid; c0 += 32u * K) {
+        uint32_t xn[K], ti[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const uint32_t c = c0 + 32u * i + lane;
+            if (c0 + 32u * i < n_valid) {
+                // lanes past column N-1 read in bounds and are not stored
+                const uint32_t p = c + P.pos, pw = p < N ? p : p - N;
+                const uint32_t yy = (Sw[c0 + 32 * i] & P.mask) ^ S[c + 1u == N ? 0u : c + 1u];
+                const uint32_t y = yy ^ (yy << P.sh1) ^ (S[pw] >> P.sh2);
+                xn[i] = y ^ tbl(Tb, 0u, y);
+                ti[i] = temper_index(S[pw ? pw - 1u : N - 1u]);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const uint32_t c = c0 + 32u * i + lane;
+            if (c < n_valid) {
+                S[c] = xn[i];
+                if (SLOW)
+                    slow_store(temper_convert<0>(xn[i], ti[i], Tb), temper_convert<1>(xn[i], ti[i], Tb),
+                               row_g + c, segs, s_first, s_end, out);
+                else
+                    __stcs(ow + c0 + 32 * i, temper_convert<FMT>(xn[i], ti[i], Tb));
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// Advances one stream whose N - pos >= 256 by the segments [s_begin, s_end),
+// this warp alone.
+template <int M>
+__device__ __forceinline__ void run_item_late(const KParams& KP, const RowP& P, uint32_t* __restrict__ g,
+                                              uint32_t* __restrict__ S, const Segment* __restrict__ segs,
+                                              uint32_t s_begin, uint32_t s_end, uint32_t* __restrict__ out,
+                                              uint32_t lane, const uint32_t* __restrict__ Tb)
+{
+    const uint32_t N = P.n;
+    for (uint32_t c = lane; c < (KP.np >> 2); c += 32u)
+        cp_async16(S + 4u * c, g + 4u * c);
+    const Segment last = segs[s_end - 1u];
+    uint32_t s = s_begin;
+    Segment sg = segs[s];
+    cp_async_wait_all();
+    __syncwarp();
+    const uint64_t total = last.g_start + last.count;
+    uint64_t seg_end = sg.g_start + sg.count;
+    uint64_t row = 0;
+    while (row < total) {
+        while (row >= seg_end) {
+            sg = segs[++s];
+            seg_end = sg.g_start + sg.count;
+        }
+        uint32_t* ow = out + sg.out_off + (row - sg.g_start) + lane;
+        if (row + N <= seg_end) {
+            // the rows that lie wholly inside this request, back to back
+            const uint32_t nfull = (uint32_t)min((seg_end - row) / N, (uint64_t)0xFFFFFFFFu);
+            if (sg.fmt == 0)
+                gen_rows_late<M, 0>(S, ow, P, lane, Tb, nfull);
+            else if (sg.fmt == 1)
+                gen_rows_late<M, 1>(S, ow, P, lane, Tb, nfull);
+            else
+                gen_rows_late<M, 2>(S, ow, P, lane, Tb, nfull);
+            row += (uint64_t)nfull * N;
+        } else {
+            const uint64_t left = total - row;
+            const uint32_t n_valid = left < (uint64_t)N ? (uint32_t)left : N;
+            if (total > seg_end)   // crosses into the next request
+                gen_row_part<M, 0, true>(S, ow, P, lane, Tb, n_valid, row, segs, s, s_end, out);
+            else if (sg.fmt == 0)
+                gen_row_part<M, 0, false>(S, ow, P, lane, Tb, n_valid, row, segs, s, s_end, out);
+            else if (sg.fmt == 1)
+                gen_row_part<M, 1, false>(S, ow, P, lane, Tb, n_valid, row, segs, s, s_end, out);
+            else
+                gen_row_part<M, 2, false>(S, ow, P, lane, Tb, n_valid, row, segs, s, s_end, out);
+            row += N;
+        }
+    }
+    // stage out: oldest word first (see run_item)
+    const uint32_t phase = (uint32_t)(total % N);
+    for (uint32_t j = lane; j < N; j += 32u) {
+        uint32_t c = phase + j;
+        c = c >= N ? c - N : c;
+        g[j] = S[c];
+    }
+    __syncwarp();
 }
 
 // Advances one stream by the segments [s_begin, s_end) of the work table.
@@ -372,20 +567,7 @@ __device__ __forceinline__ void run_item(const KParams& KP, const RowP& P, uint3
             // per row only the output pointer moves.
             const uint32_t nfull = (uint32_t)min((seg_end - row) / N, (uint64_t)0xFFFFFFFFu);
             uint32_t* ow = out + sg.out_off + (row - sg.g_start) + 32u * wk + lane;
-            bool piped = false;
-            if constexpr (K == 4 && WG == 1 && M >= 9) {
-                if (N - P.pos >= 256u) {
-                    if (sg.fmt == 0)
-                        gen_rows_pipelined<M, 0>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull);
-                    else if (sg.fmt == 1)
-                        gen_rows_pipelined<M, 1>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull);
-                    else
-                        gen_rows_pipelined<M, 2>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull);
-                    piped = true;
-                }
-            }
-            if (piped) {
-            } else if (sg.fmt == 0) {
+            if (sg.fmt == 0) {
                 for (uint32_t q = 0; q < nfull; ++q, ow += N)
                     gen_row<M, K, WG, 0, false>(r, S, Sw, ow, Q, P, wk, lane, Tb, last_lane, N, row,
                                                 segs, s, s_end, out);
@@ -423,12 +605,108 @@ __device__ __forceinline__ void run_item(const KParams& KP, const RowP& P, uint3
         __syncwarp();
 }
 
+// One stream on one warp: the late-tempering loop where its 128-word steps
+// fit (N - pos >= 256), else the general one.
+template <int M, int K>
+__device__ __forceinline__ void run_single(const KParams& KP, const RowP& P, uint32_t* __restrict__ g,
+                                           uint32_t* __restrict__ S, const Segment* __restrict__ segs,
+                                           uint32_t s_begin, uint32_t s_end, uint32_t* __restrict__ out,
+                                           uint32_t warp, uint32_t lane, const uint32_t* __restrict__ Tb)
+{
+    if constexpr (K == 4 && M >= 9) {
+        if (P.n - P.pos >= 256u) {
+            run_item_late<M>(KP, P, g, S, segs, s_begin, s_end, out, lane, Tb);
+            return;
+        }
+    }
+    run_item<M, K, 1>(KP, P, g, S, segs, s_begin, s_end, out, warp, lane, Tb);
+}
+
+// Claims.  The n items (longest first) are dealt to n_groups lists, one per
+// SM, in snake order: list g's k-th item is k n_groups + g for even k and
+// k n_groups + (n_groups - 1 - g) for odd k.  A warp takes its own SM's next
+// item, and when that list is used up helps with a list that still has more
+// items than its SM has warps (those few its own warps take in one round), or
+// with a list whose SM runs no CTA of this launch.  One list for the whole
+// device let the SMs whose warps happened to be first take more of the last
+// items than others: 1024 equal streams put 8 warps on some SMs and 5 on
+// others, and 4096 at 16 warps per SM ended anywhere between 0.83 and 0.95 ms.
+constexpr uint32_t kNoItem = 0xFFFFFFFFu;
+constexpr uint32_t kPresent = 0x80000000u;   // a list's counter: its SM runs a CTA of the launch
+
+struct Claims {
+    uint32_t* counters;   // n_groups counters, each with its kPresent bit
+    uint32_t n;           // items
+    uint32_t n_groups;
+    uint32_t spare;       // warps per SM: what a present SM is left to do itself
+    uint32_t group;       // the list this warp takes from
+};
+
+__device__ __forceinline__ uint32_t list_item(uint32_t k, uint32_t g, uint32_t n_groups)
+{
+    return k * n_groups + ((k & 1u) ? n_groups - 1u - g : g);
+}
+
+// This warp's view of the lists; one warp of each CTA marks its list.
+__device__ __forceinline__ Claims claims_begin(uint32_t* counters, uint32_t n, uint32_t n_groups)
+{
+    Claims c;
+    c.counters = counters;
+    c.n = n;
+    c.n_groups = n_groups;
+    c.spare = (gridDim.x * (blockDim.x >> 5) + n_groups - 1u) / n_groups;
+    // fewer CTAs than SMs: one list per CTA
+    c.group = gridDim.x <= n_groups ? blockIdx.x : sm_id() % n_groups;
+    if (threadIdx.x == 0u)
+        atomicOr(counters + c.group, kPresent);
+    return c;
+}
+
+// The warp's next item, or kNoItem when there is none it should take.  Every
+// round either returns or finds its list used up for good (counters only
+// grow) and moves on, so the rounds are bounded by the number of lists.
+__device__ __forceinline__ uint32_t claim_item(Claims& c, uint32_t lane)
+{
+    for (;;) {
+        uint32_t k = 0;
+        if (lane == 0u)
+            k = atomicAdd(c.counters + c.group, 1u) & ~kPresent;
+        k = __shfl_sync(MTGP_FULL, k, 0);
+        const uint32_t it = list_item(k, c.group, c.n_groups);
+        if (it < c.n)
+            return it;
+        uint32_t next = kNoItem;
+        for (uint32_t b = 1u; b < c.n_groups && next == kNoItem; b += 32u) {
+            uint32_t j = c.group + b + lane;
+            j = j >= c.n_groups ? j - c.n_groups : j;
+            bool has = false;
+            if (b + lane < c.n_groups) {
+                const uint32_t v = *(volatile uint32_t*)(c.counters + j);
+                const uint32_t ahead = (v & kPresent) ? c.spare : 0u;
+                has = list_item((v & ~kPresent) + ahead, j, c.n_groups) < c.n;
+            }
+            const uint32_t B = __ballot_sync(MTGP_FULL, has);
+            if (B)
+                next = __shfl_sync(MTGP_FULL, j, __ffs(B) - 1);
+        }
+        if (next == kNoItem)
+            return kNoItem;
+        c.group = next;
+    }
+}
+
+// Resident CTAs the compiler leaves registers for: 12 warps per SM for the
+// smaller states (168 registers), 8 for the larger ones, which keep three
+// words per column group.  At 16 warps (128 registers) the late loop spilled
+// and ran at 1190 instead of 1400 Gnumbers/s (2432 equal streams, Mexp 11213).
+constexpr int fast_min_ctas(int M, int G) { return (M < 16 ? 12 : 8) / G; }
+
 // Persistent kernel.  Phase 1: the CTA claims the longest streams (items
 // [0, n_coop) of the table, sorted longest first) one at a time and its G
 // warps advance each together.  Phase 2: every warp claims the remaining
 // items [n_coop, n_items) one by one and advances each alone.
 template <int M, int K, int G>
-__global__ void __launch_bounds__(G * 32) mtgp_fast_kernel(const KParams P, uint32_t* __restrict__ states,
+__global__ void __launch_bounds__(G * 32, fast_min_ctas(M, G)) mtgp_fast_kernel(const KParams P, uint32_t* __restrict__ states,
                                                            uint32_t n_streams,
                                                            const WorkItem* __restrict__ items,
                                                            const Segment* __restrict__ segs,
@@ -437,14 +715,16 @@ __global__ void __launch_bounds__(G * 32) mtgp_fast_kernel(const KParams P, uint
                                                            uint32_t* __restrict__ out, int* __restrict__ err,
                                                            uint64_t* __restrict__ trace,
                                                            const KSet* __restrict__ sets,
-                                                           const uint32_t* __restrict__ set_of)
+                                                           const uint32_t* __restrict__ set_of,
+                                                           uint32_t n_groups)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ uint32_t s_claim;
     // Tables: Tb[0] holds the handle's set; with per-stream sets each warp
-    // loads its stream's tables into its own Tb[warp] (192-byte rows, so
-    // every table starts on a 64-byte boundary: entry k in bank k).
-    __shared__ __align__(64) uint32_t Tb[G][48];
+    // loads its stream's tables into its own Tb[warp] (256-byte rows: every
+    // table is 64-byte aligned, entry k in bank k, and temper_addr needs the
+    // row's address to end in a zero byte).
+    __shared__ __align__(256) uint32_t Tb[G][64];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = threadIdx.x >> 5;
     if (threadIdx.x < 16) {
@@ -460,7 +740,7 @@ __global__ void __launch_bounds__(G * 32) mtgp_fast_kernel(const KParams P, uint
     // set; otherwise every item is a single-warp item.
     const uint32_t first_single = (K >= G && !sets) ? n_coop : 0u;
     if constexpr (K >= G) {
-    for (; !sets;) {
+    while (n_coop != 0u && !sets) {
         if (threadIdx.x == 0)
             s_claim = atomicAdd(&counters[0], 1u);
         __syncthreads();
@@ -483,13 +763,25 @@ __global__ void __launch_bounds__(G * 32) mtgp_fast_kernel(const KParams P, uint
     }
 
     uint32_t* S = smem + warp * fast_smem_words(P.n, P.mirror);
-    for (;;) {
-        uint32_t it = 0;
-        if (lane == 0)
-            it = first_single + atomicAdd(&counters[1], 1u);
-        it = __shfl_sync(MTGP_FULL, it, 0);
-        if (it >= n_items)
-            break;
+    // No more items than warps: each warp has its item by its place, one warp
+    // of every CTA before a second one of any, and no counter is touched.
+    const bool placed = first_single == 0u && items_placed(n_items, gridDim.x, G);
+    Claims claims;
+    if (!placed)
+        claims = claims_begin(counters + 1, n_items - first_single, n_groups);
+    for (bool more = true; more;) {
+        uint32_t it;
+        if (placed) {
+            it = warp * gridDim.x + blockIdx.x;
+            more = false;
+            if (it >= n_items)
+                break;
+        } else {
+            it = claim_item(claims, lane);
+            if (it == kNoItem)
+                break;
+            it += first_single;
+        }
         const WorkItem w = items[it];
         if (w.stream >= n_streams || w.nseg == 0) {
             if (lane == 0)
@@ -507,11 +799,11 @@ __global__ void __launch_bounds__(G * 32) mtgp_fast_kernel(const KParams P, uint
                 Tb[warp][32u + lane] = ks.flt[lane];
             }
             __syncwarp();
-            run_item<M, K, 1>(P, R, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
-                              w.seg_begin + w.nseg, out, warp, lane, Tb[warp]);
+            run_single<M, K>(P, R, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
+                             w.seg_begin + w.nseg, out, warp, lane, Tb[warp]);
         } else {
-            run_item<M, K, 1>(P, R0, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
-                              w.seg_begin + w.nseg, out, warp, lane, Tb[0]);
+            run_single<M, K>(P, R0, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
+                             w.seg_begin + w.nseg, out, warp, lane, Tb[0]);
         }
         if (trace && lane == 0)
             trace_item(trace, it, t0, segs, w);

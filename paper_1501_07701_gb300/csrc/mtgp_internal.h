@@ -65,6 +65,7 @@ struct LaunchCfg {
     int kernel;          // 0 register-resident, 1 shared-memory ring
     int coop_percent;    // streams longer than coop_percent/100 x (numbers per warp
                          // slot) are advanced by a whole CTA; 0 = never
+    bool automatic;      // the default: fit_config chooses warps for each launch's work
 };
 
 // Per-warp shared-memory footprint (32-bit words).
@@ -96,6 +97,20 @@ cudaError_t allow_max_dynamic_smem(const void* fn, int device, size_t need);
 cudaError_t launch_init(const KParams& P, const uint32_t* d_seeds, uint32_t n_streams,
                         uint32_t* d_states, cudaStream_t s);
 
+// Claim counters at the head of a work table: counters[0] for the items that
+// whole CTAs take, counters[1 + g] for group g of the others (see claim_item
+// in mtgp_fast.cuh).  Zeroed before every launch.
+constexpr uint32_t kCounterBytes = 1024;
+constexpr uint32_t kMaxGroups = kCounterBytes / 4u - 1u;
+
+// True if a launch of the register-resident kernel gives its items (none of
+// them CTA-wide) to warps by their place; it then neither reads nor needs the
+// counters.
+__host__ __device__ inline bool items_placed(uint32_t n_items, uint32_t grid, uint32_t warps)
+{
+    return (uint64_t)n_items <= (uint64_t)grid * warps;
+}
+
 struct GenArgs {
     KParams P;
     uint32_t* states;
@@ -104,7 +119,7 @@ struct GenArgs {
     const Segment* segs;
     uint32_t n_items;
     uint32_t n_coop;     // items [0, n_coop) are advanced by whole CTAs
-    uint32_t* counter;   // two claim counters, zeroed before the launch
+    uint32_t* counter;   // claim counters, zeroed before the launch
     uint32_t* out;
     int* err;
     uint64_t* trace;     // optional: 4 words per item (start ns, end ns, SM, numbers)
@@ -136,6 +151,7 @@ struct Geometry {
     int grid;
     int regs;            // registers per thread of the kernel used
     int per_sm;          // resident CTAs per SM (occupancy, after the cap)
+    int sms;             // SMs of the device
 };
 
 // Works out kernel choice, block size, shared memory and grid (persistent:
@@ -151,12 +167,12 @@ cudaError_t launch_generate(const GenArgs& a, const Geometry& g, cudaStream_t s)
 // M = ceil(N / 32) register columns per lane; returns cudaErrorInvalidValue
 // if M or K has no instantiation.
 cudaError_t launch_fast(int M, int K, int G, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
-                        cudaStream_t s);
+                        uint32_t sms, cudaStream_t s);
 const void* fast_kernel_ptr(int M, int K, int G);
 
 // Launches a generation kernel with the register-resident kernel's signature.
 cudaError_t launch_gen_fn(const void* fn, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
-                          cudaStream_t s);
+                          uint32_t sms, cudaStream_t s);
 
 // Statistics of the paper's gap test (test 35) and Hamming-weight
 // independence test (test 100), Sec. 4.2, accumulated by the fused

@@ -298,6 +298,7 @@ cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_ite
     const long long want = ((long long)n_items + warps - 1) / warps;
     const long long cap = (long long)sms * per_sm;
     g->grid = (int)std::max(1LL, std::min(want, cap));
+    g->sms = sms;
     return cudaSuccess;
 }
 
@@ -307,7 +308,7 @@ cudaError_t launch_generate(const GenArgs& a, const Geometry& g, cudaStream_t s)
         return cudaSuccess;
     if (g.kernel == 0)
         return launch_fast((int)((a.P.n + 31u) / 32u), g.k, g.threads / 32, a, dim3(g.grid),
-                           dim3(g.threads), g.smem, s);
+                           dim3(g.threads), g.smem, (uint32_t)g.sms, s);
     mtgp_ring_kernel<<<g.grid, g.threads, g.smem, s>>>(a.P, a.states, a.n_streams, a.items, a.segs,
                                                        a.n_items, a.counter, a.out, a.err, a.sets,
                                                        a.set_of);
@@ -336,16 +337,16 @@ const void* fast_kernel_ptr(int M, int K, int G)
 }
 
 cudaError_t launch_fast(int M, int K, int G, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
-                        cudaStream_t s)
+                        uint32_t sms, cudaStream_t s)
 {
     const void* fn = fast_kernel_ptr(M, K, G);
     if (!fn)
         return cudaErrorInvalidValue;
-    return launch_gen_fn(fn, a, grid, block, smem, s);
+    return launch_gen_fn(fn, a, grid, block, smem, sms, s);
 }
 
 cudaError_t launch_gen_fn(const void* fn, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
-                          cudaStream_t s)
+                          uint32_t sms, cudaStream_t s)
 {
     KParams P = a.P;
     uint32_t* states = a.states;
@@ -360,8 +361,9 @@ cudaError_t launch_gen_fn(const void* fn, const GenArgs& a, dim3 grid, dim3 bloc
     uint64_t* trace = a.trace;
     const KSet* sets = a.sets;
     const uint32_t* set_of = a.set_of;
+    uint32_t n_groups = std::max(1u, std::min(std::min(grid.x, sms), kMaxGroups));
     void* args[] = {&P, &states, &n_streams, &items, &segs, &n_items, &n_coop, &counter, &out, &err,
-                    &trace, &sets, &set_of};
+                    &trace, &sets, &set_of, &n_groups};
     return cudaLaunchKernel(fn, grid, block, args, smem, s);
 }
 

@@ -34,10 +34,10 @@ using namespace mtgp;
 namespace {
 
 // Largest request list one call accepts.  The table holds the two claim
-// counters (256 bytes, cleared on every call), one 16-byte item per
+// counters (kCounterBytes, cleared on every call), one 16-byte item per
 // distinct stream and one 32-byte segment per request.
 constexpr uint32_t kMaxRequests = 1024;
-constexpr size_t kCountersBytes = 256;
+constexpr size_t kCountersBytes = kCounterBytes;
 constexpr size_t kItemsBytes = kMaxRequests * sizeof(WorkItem);
 constexpr size_t kScratchBytes = kCountersBytes + kItemsBytes + kMaxRequests * sizeof(Segment);
 
@@ -179,7 +179,8 @@ extern "C" mtgp_status mtgp_generate_noalloc(mtgp_streams_t st, const uint32_t* 
     }
 
     Geometry g;
-    mtgp_status s = geometry_for(st, st->cfg, n_items, &g);
+    const LaunchCfg run = fit_config(st, st->cfg, n_items, total, T.item_total[0]);
+    mtgp_status s = geometry_for(st, run, n_items, &g);
     if (s != MTGP_OK)
         return s;
     // Longest streams to whole CTAs, as in the ordinary path.

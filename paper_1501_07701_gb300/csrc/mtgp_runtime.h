@@ -3,6 +3,7 @@
 #pragma once
 
 #include <array>
+#include <map>
 #include <new>
 #include <tuple>
 #include <vector>
@@ -75,10 +76,9 @@ struct mtgp_streams {
     mtgp::LaunchCfg cfg{};
     std::array<mtgp::TableSlot, 4> slots{};
     int next_slot = 0;
-    // launch geometry cache (for the current cfg; grid = residency cap)
-    bool geo_valid = false;
-    std::tuple<int, int, int, int> geo_key{};
-    mtgp::Geometry geo_cap{};
+    // launch geometry per configuration (warps per CTA, CTAs per SM, sub-steps,
+    // kernel; grid = residency cap)
+    std::map<std::tuple<int, int, int, int>, mtgp::Geometry> geo_caps;
     // device-to-host path
     // (kStages buffers: generation may run that many chunks ahead of the copies)
     static constexpr int kStages = 4;
@@ -91,6 +91,7 @@ struct mtgp_streams {
     // together before its first kernel
     void* d_chunk_tables = nullptr;
     size_t chunk_tables_cap = 0;
+    int sms = 1;              // SMs of the device
     // autotuning
     cudaStream_t tune_stream = nullptr;
     cudaEvent_t tune_ev[2] = {nullptr, nullptr};
@@ -187,6 +188,11 @@ mtgp_status build_work(uint32_t n_streams, const uint32_t* ids, const uint64_t* 
 size_t table_bytes(const Work& w, size_t* items_off, size_t* segs_off);
 void fill_table(const Work& w, void* host);
 LaunchCfg default_config(const KParams& P);
+// The configuration a launch of this work runs with: `cfg` itself, or for the
+// default configuration its warps per CTA and CTAs per SM chosen from the
+// number of items, their total and the longest.
+LaunchCfg fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
+                     uint64_t max_item);
 mtgp_status geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, Geometry* g);
 mtgp_status launch_work(mtgp_streams* st, const Work& w, const LaunchCfg& cfg, void* out,
                         cudaStream_t s);
