@@ -31,6 +31,8 @@
 // barrier, then writes everything.
 #pragma once
 
+#include <utility>
+
 #include "mtgp_internal.h"
 
 namespace mtgp {
@@ -271,36 +273,55 @@ __device__ __forceinline__ void gen_row(uint32_t (&r)[(M + WG - 1) / WG], uint32
 // 11.4 ALU instructions per 32 numbers, LSU data stage 85 % and ALU 74 % busy
 // (the loop it replaced: 7.34 and 13.3).  Hence the late tempering and the
 // wrapped addresses (LSU), the packed folds and the multiply for the left
-// shift (ALU).  The rows are unrolled because a row of three steps leaves its
-// pointer and register moves exposed: one stream alone took 0.62 ms for 2^20
-// numbers with one row per pass, 0.51 with four.  All together: the uneven
-// workload 4.72 -> 3.61 ms (1085 -> 1419 Gnumbers/s, 0.84 of the HBM rate),
-// 4096 x 2^18 at 12 warps per SM 1.02 -> 0.79 ms, one stream of 2^20 numbers
-// 0.75 -> 0.51 ms; Mexp 44497, 1024 x 2^20, 1.15 -> 0.95 ms.
+// shift (ALU).  Only the packed tempering indices are kept for a row, a
+// quarter register per column group: kept table words made the 44 groups of
+// Mexp 44497 spill (0.98 against 0.86 ms).  The rows are unrolled because a
+// row of three steps leaves its pointer and register moves exposed: one
+// stream alone took 0.62 ms for 2^20 numbers with one row per pass, 0.52 with
+// four.  All together: the uneven workload 4.72 -> 3.60 ms (1085 -> 1422
+// Gnumbers/s, 0.84 of the HBM rate), 4096 x 2^18 at 12 warps per SM 1.02 ->
+// 0.79 ms, one stream of 2^20 numbers 0.75 -> 0.52 ms; Mexp 44497, 1024 x
+// 2^20, 1.15 -> 0.86 ms.
 // ===========================================================================
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t lds(uint32_t a)
+// Shared loads and stores at a compile-time offset from a 32-bit shared
+// address: the offset is part of the instruction, so one address register
+// serves a whole row.
+template <int OFF>
+__device__ __forceinline__ uint32_t lds_at(uint32_t a)
 {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF) : "memory");
     return v;
 }
-__device__ __forceinline__ void sts(uint32_t a, uint32_t v)
+template <int OFF>
+__device__ __forceinline__ void sts_at(uint32_t a, uint32_t v)
 {
-    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+    asm volatile("st.shared.u32 [%0+%1], %2;" ::"r"(a), "n"(OFF), "r"(v) : "memory");
 }
-// Table addresses (less the table's offset) of four tempering words at once:
-// their 16-bit and 8-bit folds run packed, two and four words to a register,
-// and one byte permute per word then puts 4 * index under the table base tb,
-// a multiple of 256.  13 ALU instructions for four words, 16 one by one.
-__device__ __forceinline__ void temper_addr(const uint32_t (&x)[4], uint32_t tb, uint32_t (&a)[4])
+
+// f(0), f(1), .. f(N-1), the argument a compile-time constant.
+template <class F, int... I>
+__device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, I...>)
+{
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F&& f)
+{
+    static_for_impl(f, std::make_integer_sequence<int, N>{});
+}
+
+// Tempering indices of four words at once, as bytes 4 * index: the 16-bit and
+// 8-bit folds run packed, two and four words to a register.  A byte permute
+// then puts one of them under the table base tb, a multiple of 256, as the
+// lookup's address (less the table's offset).  13 ALU instructions for four
+// words in all, 16 one by one.
+__device__ __forceinline__ uint32_t temper_pack(const uint32_t (&x)[4])
 {
     const uint32_t u = __byte_perm(x[0], x[1], 0x5410) ^ __byte_perm(x[0], x[1], 0x7632);
     const uint32_t v = __byte_perm(x[2], x[3], 0x5410) ^ __byte_perm(x[2], x[3], 0x7632);
-    const uint32_t w = ((__byte_perm(u, v, 0x6420) ^ __byte_perm(u, v, 0x7531)) & 0x0F0F0F0Fu) * 4u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        a[i] = __byte_perm(w, tb, 0x7650 + i);
+    return ((__byte_perm(u, v, 0x6420) ^ __byte_perm(u, v, 0x7531)) & 0x0F0F0F0Fu) * 4u;
 }
 
 template <int FMT>
@@ -321,6 +342,7 @@ __device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const R
     constexpr int K = 4;
     constexpr int NS = (M + K - 1) / K;   // steps per row (>= 3 here)
     constexpr int U = NS <= 3 ? 4 : 2;    // rows per pass of the unrolled loop
+    constexpr int TT = FMT == 0 ? 64 : 128;   // byte offset of the tempering table
     const uint32_t N = P.n, last_lane = (N - 1u) & 31u;   // lane of column N-1 (group M-1)
     uint32_t sa = saddr(S + lane);
     uint32_t x1_last = lane >= last_lane ? saddr(S) : sa + 128u * (M - 1) + 4u;
@@ -329,80 +351,85 @@ __device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const R
     // see through: the FMA pipe is idle, the ALU pipe is not
     uint32_t mul1 = 1u << P.sh1;
     asm volatile("" : "+r"(mul1), "+r"(sa), "+r"(x1_last), "+r"(tb));
-    uint32_t r[M], qa[M], T[M];
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        const uint32_t p = 32u * (uint32_t)m + lane + P.pos;
-        r[m] = lds(sa + 128u * m);
+    uint32_t r[M], qa[M];
+    uint32_t T[NS];   // the steps' tempering indices, packed
+    static_for<M>([&](auto im) {
+        constexpr int m = im.value;
+        const uint32_t p = 32u * m + lane + P.pos;
+        r[m] = lds_at<128 * m>(sa);
         qa[m] = saddr(S + (p < N ? p : p - N));
         asm volatile("" : "+r"(qa[m]));   // kept, not worked out again in the loop
-        T[m] = 0u;
-    }
-    T[M - 1] = tbl(Tb, FMT == 0 ? 16u : 32u, temper_index(S[P.pos - 1u]));
+    });
+    static_for<NS>([&](auto is) { T[is.value] = 0u; });
+    T[NS - 1] = (temper_index(S[P.pos - 1u]) & 15u) << (2 + 8 * ((M - 1) & 3));
     uint32_t x1[K], xp[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-        x1[i] = lds(sa + 128u * i + 4u);
-        xp[i] = lds(qa[i]);
-    }
+    static_assert(M >= K, "step 0 fills all of x1 and xp");
+    static_for<K>([&](auto ii) {
+        constexpr int i = ii.value;
+        x1[i] = lds_at<128 * i + 4>(sa);
+        xp[i] = lds_at<0>(qa[i]);
+    });
     uint32_t* op = ow + 1 - (int)N;   // where column `lane` of this row stores
 #pragma unroll U
     for (uint32_t q = 0; q < nfull; ++q, op += N) {
         const bool body = q != 0u;
         const bool last = lane == last_lane || (body && lane < last_lane);
-#pragma unroll
-        for (int st = 0; st < NS; ++st) {
-            const int s0 = st * K;
-            const int n0 = (st + 1 < NS) ? s0 + K : 0;   // next step (next row's first)
-            uint32_t y1[K], yp[K];
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                if (n0 + i < M) {
-                    y1[i] = n0 + i + 1 < M ? lds(sa + 128u * (n0 + i) + 4u) : lds(x1_last);
-                    yp[i] = lds(qa[n0 + i]);
+        static_for<NS>([&](auto is) {
+            constexpr int st = is.value, s0 = st * K;
+            constexpr int n0 = (st + 1 < NS) ? s0 + K : 0;   // next step (next row's first)
+            uint32_t y1[K], yp[K], xn[K], o[K], tw[K];
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value, m = n0 + i;
+                if constexpr (m < M) {
+                    if constexpr (m + 1 < M)
+                        y1[i] = lds_at<128 * m + 4>(sa);
+                    else
+                        y1[i] = lds_at<0>(x1_last);
+                    yp[i] = lds_at<0>(qa[m]);
                 }
-            }
-            uint32_t ta[K];
-            temper_addr(xp, tb, ta);
-            uint32_t xn[K], o[K];
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const int m = s0 + i;
-                if (m < M) {
+            });
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value;
+                if constexpr (s0 + i < M)
+                    tw[i] = lds_at<TT>(__byte_perm(T[st], tb, 0x7650 + i));
+            });
+            T[st] = temper_pack(xp);
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value, m = s0 + i;
+                if constexpr (m < M) {
                     const uint32_t yy = (r[m] & P.mask) ^ x1[i];
                     const uint32_t y = yy ^ (yy * mul1) ^ (xp[i] >> P.sh2);
                     xn[i] = y ^ tbl(Tb, 0u, y);
-                    o[i] = finish<FMT>(x1[i], T[m]);
-                    T[m] = lds(ta[i] + (FMT == 0 ? 64u : 128u));
+                    o[i] = finish<FMT>(x1[i], tw[i]);
                 }
-            }
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const int m = s0 + i;
-                if (m < M) {
+            });
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value, m = s0 + i;
+                if constexpr (m < M) {
                     r[m] = xn[i];
-                    sts(sa + 128u * m, xn[i]);
+                    sts_at<128 * m>(sa, xn[i]);
                     if (m + 1 < M ? body : last)
                         __stcs(op + 32 * m, o[i]);
                 }
-            }
+            });
             __syncwarp();
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                if (n0 + i < M) {
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value;
+                if constexpr (n0 + i < M) {
                     x1[i] = y1[i];
                     xp[i] = yp[i];
                 }
-            }
-        }
+            });
+        });
     }
     // the last row's numbers after its first
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        const uint32_t v = lds(sa + 128u * m + 4u);
+    static_for<M>([&](auto im) {
+        constexpr int m = im.value;
+        const uint32_t v = lds_at<128 * m + 4>(sa);
+        const uint32_t tw = lds_at<TT>(__byte_perm(T[m / K], tb, 0x7650 + m % K));
         if (m + 1 < M || lane < last_lane)
-            __stcs(op + 32 * m, finish<FMT>(v, T[m]));
-    }
+            __stcs(op + 32 * m, finish<FMT>(v, tw));
+    });
 }
 
 // A row on the same layout (no mirror) with its numbers stored at once:
@@ -699,14 +726,19 @@ __device__ __forceinline__ uint32_t claim_item(Claims& c, uint32_t lane)
 // smaller states (168 registers), 8 for the larger ones, which keep three
 // words per column group.  At 16 warps (128 registers) the late loop spilled
 // and ran at 1190 instead of 1400 Gnumbers/s (2432 equal streams, Mexp 11213).
-constexpr int fast_min_ctas(int M, int G) { return (M < 16 ? 12 : 8) / G; }
+// The other row loops need few registers and gain from many warps: 16 per SM,
+// 32 for short states.
+constexpr int fast_min_ctas(int M, int K, int G)
+{
+    return (M < 9 ? 32 : K != 4 ? 16 : M < 16 ? 12 : 8) / G;
+}
 
 // Persistent kernel.  Phase 1: the CTA claims the longest streams (items
 // [0, n_coop) of the table, sorted longest first) one at a time and its G
 // warps advance each together.  Phase 2: every warp claims the remaining
 // items [n_coop, n_items) one by one and advances each alone.
 template <int M, int K, int G>
-__global__ void __launch_bounds__(G * 32, fast_min_ctas(M, G)) mtgp_fast_kernel(const KParams P, uint32_t* __restrict__ states,
+__global__ void __launch_bounds__(G * 32, fast_min_ctas(M, K, G)) mtgp_fast_kernel(const KParams P, uint32_t* __restrict__ states,
                                                            uint32_t n_streams,
                                                            const WorkItem* __restrict__ items,
                                                            const Segment* __restrict__ segs,
