@@ -293,8 +293,10 @@ extern "C" mtgp_status mtgp_params_free(mtgp_params_t params)
 // ---------------------------------------------------------------------------
 mtgp_status mtgp::build_work(uint32_t n_streams, const uint32_t* ids, const uint64_t* counts,
                              const int32_t* fmts, uint32_t fmt_all, uint32_t n_req,
-                             uint64_t out_base, Work& w, const uint64_t* out_offs)
+                             uint64_t out_base, Work& w, const uint64_t* out_offs, BuildScratch* scratch)
 {
+    BuildScratch own;
+    BuildScratch& b = scratch ? *scratch : own;
     w.items.clear();
     w.item_total.clear();
     w.segs.clear();
@@ -304,9 +306,13 @@ mtgp_status mtgp::build_work(uint32_t n_streams, const uint32_t* ids, const uint
         return MTGP_OK;
     if (!ids || !counts)
         return fail(MTGP_EINVAL, "null request arrays");
-    std::vector<uint32_t> order;
-    order.reserve(n_req);
+    b.order.clear();
+    b.off.resize(n_req);
+    // exclusive scan of counts in request order gives the output offsets
+    // (unless the caller places every request itself)
     uint64_t total = 0;
+    bool ascending = true;   // the ids of the requests with numbers, strictly
+    uint32_t last_id = 0;
     for (uint32_t j = 0; j < n_req; ++j) {
         if (ids[j] >= n_streams)
             return fail(MTGP_EINVAL, "stream id %u >= n_streams %u (request %u)", ids[j], n_streams, j);
@@ -314,62 +320,70 @@ mtgp_status mtgp::build_work(uint32_t n_streams, const uint32_t* ids, const uint
             return fail(MTGP_EINVAL, "format %d of request %u", fmts[j], j);
         if (counts[j] > (1ull << 50) || total + counts[j] < total)
             return fail(MTGP_EINVAL, "count too large (request %u)", j);
+        b.off[j] = out_offs ? out_offs[j] : out_base + total;
         total += counts[j];
-        if (counts[j])
-            order.push_back(j);
+        if (counts[j]) {
+            ascending = ascending && (b.order.empty() || ids[j] > last_id);
+            last_id = ids[j];
+            b.order.push_back(j);
+        }
     }
-    std::stable_sort(order.begin(), order.end(),
-                     [&](uint32_t a, uint32_t b) { return ids[a] < ids[b]; });
-    // exclusive scan of counts in request order gives the output offsets
-    // (unless the caller places every request itself)
-    std::vector<uint64_t> off(n_req);
-    uint64_t acc = out_base;
-    for (uint32_t j = 0; j < n_req; ++j) {
-        off[j] = out_offs ? out_offs[j] : acc;
-        acc += counts[j];
-    }
+    if (!ascending)
+        std::stable_sort(b.order.begin(), b.order.end(),
+                         [&](uint32_t x, uint32_t y) { return ids[x] < ids[y]; });
+    w.segs.reserve(b.order.size());
+    w.items.reserve(b.order.size());
+    w.item_total.reserve(b.order.size());
+    bool longest_first = true;
     size_t i = 0;
-    while (i < order.size()) {
-        const uint32_t sid = ids[order[i]];
+    while (i < b.order.size()) {
+        const uint32_t sid = ids[b.order[i]];
         WorkItem it;
         it.stream = sid;
         it.seg_begin = (uint32_t)w.segs.size();
         it.pad = 0;
         uint64_t g = 0;
-        while (i < order.size() && ids[order[i]] == sid) {
-            const uint32_t j = order[i];
-            Segment s;
-            s.g_start = g;
-            s.count = counts[j];
-            s.out_off = off[j];
-            s.fmt = fmts ? (uint32_t)fmts[j] : fmt_all;
-            s.req = j;
-            w.segs.push_back(s);
+        do {
+            const uint32_t j = b.order[i];
+            w.segs.push_back(Segment{g, counts[j], b.off[j], fmts ? (uint32_t)fmts[j] : fmt_all, j});
             g += counts[j];
             ++i;
-        }
+        } while (i < b.order.size() && ids[b.order[i]] == sid);
         it.nseg = (uint32_t)w.segs.size() - it.seg_begin;
+        longest_first = longest_first && (w.items.empty() || w.item_total.back() >= g);
         w.items.push_back(it);
+        w.item_total.push_back(g);
         w.max_item = std::max(w.max_item, g);
     }
-    // Longest stream first: a warp that starts late only gets short streams.
-    std::vector<uint64_t> tot(w.items.size());
-    for (size_t k = 0; k < w.items.size(); ++k) {
-        const Segment& l = w.segs[w.items[k].seg_begin + w.items[k].nseg - 1];
-        tot[k] = l.g_start + l.count;
-    }
-    std::vector<uint32_t> idx(w.items.size());
-    for (size_t k = 0; k < idx.size(); ++k)
-        idx[k] = (uint32_t)k;
-    std::stable_sort(idx.begin(), idx.end(), [&](uint32_t a, uint32_t b) { return tot[a] > tot[b]; });
-    std::vector<WorkItem> sorted(w.items.size());
-    w.item_total.resize(w.items.size());
-    for (size_t k = 0; k < idx.size(); ++k) {
-        sorted[k] = w.items[idx[k]];
-        w.item_total[k] = tot[idx[k]];
-    }
-    w.items.swap(sorted);
     w.total = total;
+    if (longest_first)
+        return MTGP_OK;
+    // Longest stream first: a warp that starts late only gets short streams.
+    // (Equal ones keep their order.)
+    const size_t n = w.items.size();
+    b.idx.resize(n);
+    if (w.max_item < (1ull << 32)) {
+        // one 64-bit key per item: the complement of its length, then its place
+        b.keys.resize(n);
+        for (size_t k = 0; k < n; ++k)
+            b.keys[k] = (uint64_t)(uint32_t)~(uint32_t)w.item_total[k] << 32 | k;
+        std::sort(b.keys.begin(), b.keys.end());
+        for (size_t k = 0; k < n; ++k)
+            b.idx[k] = (uint32_t)b.keys[k];
+    } else {
+        for (size_t k = 0; k < n; ++k)
+            b.idx[k] = (uint32_t)k;
+        std::stable_sort(b.idx.begin(), b.idx.end(),
+                         [&](uint32_t x, uint32_t y) { return w.item_total[x] > w.item_total[y]; });
+    }
+    b.sorted.resize(n);
+    b.tot.resize(n);
+    for (size_t k = 0; k < n; ++k) {
+        b.sorted[k] = w.items[b.idx[k]];
+        b.tot[k] = w.item_total[b.idx[k]];
+    }
+    w.items.swap(b.sorted);
+    w.item_total.swap(b.tot);
     return MTGP_OK;
 }
 
@@ -724,6 +738,11 @@ LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_
         // 8, takes 4.3 ms at 12 and 3.6 at 8
         c.warps_per_cta = 4;
         c.ctas_per_sm = 3;
+    } else if (st->P.k.n > 1024u) {
+        // the same 8 warps as two CTAs: the 8-warp instantiation of the
+        // largest states spills (1024 x 2^20, Mexp 44497: 1.00 against 0.86 ms)
+        c.warps_per_cta = 4;
+        c.ctas_per_sm = 2;
     }
     return c;
 }
@@ -819,19 +838,12 @@ mtgp_status mtgp::launch_work(mtgp_streams* st, const Work& w, const LaunchCfg& 
     return launch_work_slot(st, sl, w, cfg, out, s);
 }
 
-// Uploads a work table through `sl` (waiting for the slot's previous
-// consumer) and launches on `s`; records the slot's event after the kernel.
-mtgp_status mtgp::launch_work_slot(mtgp_streams* st, TableSlot& sl, const Work& w,
-                                   const LaunchCfg& cfg, void* out, cudaStream_t s, const RowArray* rows)
+mtgp_status mtgp::reserve_slot(TableSlot& sl, size_t bytes)
 {
-    if (w.items.empty())
-        return MTGP_OK;
     if (sl.ev_recorded) {
         CUDA_TRY(cudaEventSynchronize(sl.ev), "cudaEventSynchronize(table slot)");
         sl.ev_recorded = false;
     }
-    size_t io, so;
-    const size_t bytes = table_bytes(w, &io, &so);
     if (bytes > sl.cap) {
         if (sl.host)
             cudaFreeHost(sl.host);
@@ -845,12 +857,42 @@ mtgp_status mtgp::launch_work_slot(mtgp_streams* st, TableSlot& sl, const Work& 
         CUDA_TRY(cudaMalloc(&sl.dev, cap), "cudaMalloc(work table)");
         sl.cap = cap;
     }
+    return MTGP_OK;
+}
+
+// Largest work table (bytes after the counters) that a launch reads from host
+// memory.
+static constexpr size_t kInPlaceTable = 16384;
+
+// Hands a work table to a launch through `sl` (waiting for the slot's previous
+// consumer) and launches on `s`; records the slot's event after the kernel.
+mtgp_status mtgp::launch_work_slot(mtgp_streams* st, TableSlot& sl, const Work& w,
+                                   const LaunchCfg& cfg, void* out, cudaStream_t s, const RowArray* rows)
+{
+    if (w.items.empty())
+        return MTGP_OK;
+    size_t io, so;
+    const size_t bytes = table_bytes(w, &io, &so);
+    mtgp_status r = reserve_slot(sl, bytes);
+    if (r != MTGP_OK)
+        return r;
     fill_table(w, sl.host);
-    CUDA_TRY(cudaMemcpyAsync(sl.dev, sl.host, bytes, cudaMemcpyHostToDevice, s),
-             "cudaMemcpyAsync(work table)");
-    mtgp_status stt = launch_work_table(st, w, sl.dev, cfg, out, s, rows);
-    if (stt != MTGP_OK)
-        return stt;
+    const LaunchCfg run = fit_config(st, cfg, (uint32_t)w.items.size(), w.total, w.max_item);
+    Geometry g;
+    r = geometry_for(st, run, (uint32_t)w.items.size(), &g);
+    if (r != MTGP_OK)
+        return r;
+    // A launch whose items are placed reads each entry of the table once and
+    // needs no counters, so a small table stays in the pinned host buffer and
+    // the warps read it there: no copy for the kernel to wait for.
+    const bool in_place = bytes <= kCounterBytes + kInPlaceTable && g.kernel == 0 && run.coop_percent == 0 &&
+                          items_placed((uint32_t)w.items.size(), (uint32_t)g.grid, (uint32_t)g.threads / 32u);
+    if (!in_place)
+        CUDA_TRY(cudaMemcpyAsync(sl.dev, sl.host, bytes, cudaMemcpyHostToDevice, s),
+                 "cudaMemcpyAsync(work table)");
+    r = launch_work_table(st, w, in_place ? sl.host : sl.dev, run, out, s, rows);
+    if (r != MTGP_OK)
+        return r;
     CUDA_TRY(cudaEventRecord(sl.ev, s), "cudaEventRecord");
     sl.ev_recorded = true;
     return MTGP_OK;
@@ -899,8 +941,9 @@ static mtgp_status generate_common(mtgp_streams_t st, const uint32_t* ids, const
         return fail(MTGP_EINVAL, "null handle");
     if (fmt > 2)
         return fail(MTGP_EINVAL, "format %u", fmt);
-    Work w;
-    mtgp_status s = build_work(st->n_streams, ids, counts, nullptr, fmt, n_req, 0, w);
+    Work& w = st->call_work;
+    mtgp_status s = build_work(st->n_streams, ids, counts, nullptr, fmt, n_req, 0, w, nullptr,
+                               &st->call_scratch);
     if (s != MTGP_OK)
         return s;
     if (w.total && !out)

@@ -30,6 +30,14 @@ struct Work {
     uint64_t max_item = 0;
 };
 
+// Host arrays of build_work that a handle keeps between calls.
+struct BuildScratch {
+    std::vector<uint32_t> order, idx;
+    std::vector<uint64_t> off, keys;
+    std::vector<WorkItem> sorted;
+    std::vector<uint64_t> tot;
+};
+
 // A pinned host buffer and a device buffer holding one uploaded work table
 // (work counter, items, segments); `ev` marks the end of the kernel that
 // consumed it, so the slot can be refilled.
@@ -92,6 +100,9 @@ struct mtgp_streams {
     void* d_chunk_tables = nullptr;
     size_t chunk_tables_cap = 0;
     int sms = 1;              // SMs of the device
+    // the direct calls' work and its scratch (calls on one handle do not overlap)
+    mtgp::Work call_work;
+    mtgp::BuildScratch call_scratch;
     // autotuning
     cudaStream_t tune_stream = nullptr;
     cudaEvent_t tune_ev[2] = {nullptr, nullptr};
@@ -184,7 +195,7 @@ namespace mtgp {
 // to out_base + the exclusive prefix sum of counts.
 mtgp_status build_work(uint32_t n_streams, const uint32_t* ids, const uint64_t* counts,
                        const int32_t* fmts, uint32_t fmt_all, uint32_t n_req, uint64_t out_base,
-                       Work& w, const uint64_t* out_offs = nullptr);
+                       Work& w, const uint64_t* out_offs = nullptr, BuildScratch* scratch = nullptr);
 size_t table_bytes(const Work& w, size_t* items_off, size_t* segs_off);
 void fill_table(const Work& w, void* host);
 LaunchCfg default_config(const KParams& P);
@@ -211,6 +222,8 @@ mtgp_status launch_work_slot(mtgp_streams* st, TableSlot& sl, const Work& w, con
 mtgp_status launch_work_table(mtgp_streams* st, const Work& w, void* table, const LaunchCfg& cfg,
                               void* out, cudaStream_t s, const RowArray* rows = nullptr);
 void free_table_slot(TableSlot& s);
+// Waits for the slot's previous consumer and makes room for `bytes`.
+mtgp_status reserve_slot(TableSlot& s, size_t bytes);
 mtgp_status validate_config(const mtgp_launch_config* c, LaunchCfg* out);
 // Number of leading (longest) items a launch hands to whole CTAs.
 uint32_t coop_count(const Work& w, const Geometry& g, int coop_percent);
