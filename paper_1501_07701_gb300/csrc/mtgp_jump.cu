@@ -24,15 +24,19 @@
 // windows of its share of g's set bits into the N-word accumulator, and the
 // last step is applied to the result.
 #include <algorithm>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <random>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "../../include/mtgp_mt.h"
 #include "mtgp_runtime.h"
 
 using namespace mtgp;
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -377,18 +381,100 @@ const Poly* cached_mu(const Rec& p, uint32_t mexp)
 }
 
 // ---------------------------------------------------------------------------
-// Device: one CTA per (stream, jump).  Shared memory: the sequence S[0 .. D+N-1)
-// and the N-word accumulator.  Every wait is a __syncthreads on uniform
-// control flow; no spin waits.
+// Device: one CTA, or a cluster of up to 8, per (stream, jump).  Shared memory
+// of each CTA: the N-word accumulator, then the sequence S[0 .. D+N-1).  Every
+// wait is a CTA or cluster barrier on uniform control flow; no spin waits.
+//
+// Accumulation, acc[c] = XOR over the set bits k of g of S[k + c].  Bits k of
+// one residue rho mod 32 meet the same words of a lane: with c = 32 u + lane
+// and k = 32 w + rho the word is Y[w + u], Y[v] = S[rho + 32 v + lane].  So a
+// warp takes one residue at a time, slides a window of Y through registers
+// (one shared load per 32 words and residue instead of one per set bit and 32
+// words) and applies four bits w .. w+3 at once: a 16-way branch, uniform
+// across the warp, on their pattern, each way a fixed list of three-input
+// XORs into the UC accumulators (none for pattern 0; 1.25 per accumulator and
+// four bits on average).  The bound is the ALU: about 0.31 UC D XORs per
+// lane, 38 000 warp instructions at Mexp 11213, where the shared loads of the
+// first version (one per set bit and unit, 61 000) were its bound.
+// Measured (one GB300): see launch_jump_batch.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) mtgp_jump_kernel(const KParams P, uint32_t* __restrict__ states,
-                                                       const JumpItem* __restrict__ items,
-                                                       const uint32_t* __restrict__ polys,
-                                                       uint32_t poly_words,
-                                                       const KSet* __restrict__ sets)
+constexpr int kJumpWarps = 16;
+
+// Bits P of the four bits at window position 4 G: a[u] ^= their words.
+template <int UC, int P, int G>
+__device__ __forceinline__ void jump_xor(uint32_t (&a)[UC], const uint32_t (&win)[16])
+{
+#pragma unroll
+    for (int u = 0; u < UC; ++u) {
+        uint32_t v = a[u];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if ((P >> j) & 1)
+                v ^= win[(4 * G + u + j) & 15];
+        a[u] = v;
+    }
+}
+
+template <int UC, int G>
+__device__ __forceinline__ void jump_nibble(uint32_t p, uint32_t (&a)[UC], const uint32_t (&win)[16])
+{
+    switch (p) {
+    case 1: jump_xor<UC, 1, G>(a, win); break;
+    case 2: jump_xor<UC, 2, G>(a, win); break;
+    case 3: jump_xor<UC, 3, G>(a, win); break;
+    case 4: jump_xor<UC, 4, G>(a, win); break;
+    case 5: jump_xor<UC, 5, G>(a, win); break;
+    case 6: jump_xor<UC, 6, G>(a, win); break;
+    case 7: jump_xor<UC, 7, G>(a, win); break;
+    case 8: jump_xor<UC, 8, G>(a, win); break;
+    case 9: jump_xor<UC, 9, G>(a, win); break;
+    case 10: jump_xor<UC, 10, G>(a, win); break;
+    case 11: jump_xor<UC, 11, G>(a, win); break;
+    case 12: jump_xor<UC, 12, G>(a, win); break;
+    case 13: jump_xor<UC, 13, G>(a, win); break;
+    case 14: jump_xor<UC, 14, G>(a, win); break;
+    case 15: jump_xor<UC, 15, G>(a, win); break;
+    default: break;
+    }
+}
+
+// Sixteen bits at y = &Y[w]: win holds Y[w .. w + UC - 2] on entry and
+// Y[w + 16 .. w + UC + 14] on return (position i of Y at win[i mod 16]).
+template <int UC>
+__device__ __forceinline__ void jump_block16(uint32_t bits, const uint32_t* y, uint32_t (&a)[UC],
+                                             uint32_t (&win)[16])
+{
+    static_assert(UC + 3 <= 16, "the window covers four bits and UC accumulators");
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        win[(UC - 1 + i) & 15] = y[32 * (UC - 1 + i)];
+    jump_nibble<UC, 0>(bits & 15u, a, win);
+#pragma unroll
+    for (int i = 4; i < 8; ++i)
+        win[(UC - 1 + i) & 15] = y[32 * (UC - 1 + i)];
+    jump_nibble<UC, 1>((bits >> 4) & 15u, a, win);
+#pragma unroll
+    for (int i = 8; i < 12; ++i)
+        win[(UC - 1 + i) & 15] = y[32 * (UC - 1 + i)];
+    jump_nibble<UC, 2>((bits >> 8) & 15u, a, win);
+#pragma unroll
+    for (int i = 12; i < 16; ++i)
+        win[(UC - 1 + i) & 15] = y[32 * (UC - 1 + i)];
+    jump_nibble<UC, 3>((bits >> 12) & 15u, a, win);
+}
+
+// UC: 32-word units of the accumulator that one pass covers.  s_len: words of
+// S that the launch's shared memory holds, at least D + N - 1; blocks of 32
+// bits whose window would reach past it go bit by bit.
+template <int UC>
+__global__ void __launch_bounds__(32 * kJumpWarps) mtgp_jump_kernel(
+    const KParams P, uint32_t* __restrict__ states, const JumpItem* __restrict__ items,
+    const uint32_t* __restrict__ polys, uint32_t poly_words, const KSet* __restrict__ sets, uint32_t s_len)
 {
     extern __shared__ __align__(16) uint32_t sm[];
-    const JumpItem it = items[blockIdx.x];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t part = cluster.block_rank(), parts = cluster.num_blocks();
+    const JumpItem it = items[blockIdx.x / parts];
     const uint32_t N = P.n, D = it.deg + 1u;
     uint32_t pos = P.pos, sh1 = P.sh1, sh2 = P.sh2;
     const uint32_t* rec = P.rec;
@@ -399,8 +485,8 @@ __global__ void __launch_bounds__(256) mtgp_jump_kernel(const KParams P, uint32_
         sh2 = ks.sh2;
         rec = ks.rec;
     }
-    uint32_t* S = sm;                 // D + N - 1 words
-    uint32_t* acc = sm + D + N - 1u;  // N words
+    uint32_t* acc = sm;      // N words
+    uint32_t* S = sm + N;    // s_len words, D + N - 1 of them used
     __shared__ uint32_t R[16];
     if (threadIdx.x < 16)
         R[threadIdx.x] = rec[threadIdx.x];
@@ -410,61 +496,83 @@ __global__ void __launch_bounds__(256) mtgp_jump_kernel(const KParams P, uint32_
         acc[j] = 0u;
     }
     __syncthreads();
-    // expand: S[i + N] for i = 0 .. D-2, Wc words per step, one per thread
-    // (each reads only words produced before the step: Wc <= N - pos)
+    // expand: S[i + N] for i = 0 .. D-2, Wc words per step, one per thread.
+    // A step reads only words below i0 + N, produced before it (Wc <= N - pos),
+    // and writes only words from i0 + N on: one barrier per step.
     const uint32_t Wc = min(blockDim.x, N - pos);
     for (uint32_t i0 = 0; i0 + 1u < D; i0 += Wc) {
         const uint32_t i = i0 + threadIdx.x;
-        uint32_t v = 0;
-        const bool act = threadIdx.x < Wc && i + 1u < D;
-        if (act) {
+        if (threadIdx.x < Wc && i + 1u < D) {
             uint32_t y = (S[i] & P.mask) ^ S[i + 1u];
             y ^= y << sh1;
             y ^= S[i + pos] >> sh2;
-            v = y ^ R[y & 15u];
+            S[i + N] = y ^ R[y & 15u];
         }
         __syncthreads();
-        if (act)
-            S[i + N] = v;
-        __syncthreads();
     }
-    // accumulate: warp w takes the set bits k of g with k / 32 = w (mod
-    // warps); acc[j] ^= S[k + j] for every such k.  The N words are covered
-    // in nch passes of uc <= 12 units of 32 words (one word per lane per
-    // unit), so that a pass wastes at most one unit's loads.
+    // accumulate: the workers (warps of all parts) share out the residues,
+    // or, when there are more than 32, each residue's blocks of 32 bits too
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const uint32_t* gp = polys + (size_t)it.poly * poly_words;
-    constexpr uint32_t kUnits = 12;
-    const uint32_t U = (N + 31u) / 32u;
-    const uint32_t nch = (U + kUnits - 1u) / kUnits;
-    const uint32_t uc = (U + nch - 1u) / nch;
-    for (uint32_t c = 0; c < nch; ++c) {
-        const uint32_t j0 = 32u * uc * c;
-        uint32_t a[kUnits];
+    const uint32_t workers = nw * parts, id = part * nw + warp;
+    const uint32_t nseg = workers > 32u ? workers / 32u : 1u, seg = id / 32u;
+    const uint32_t W = (D + 31u) / 32u, nb = (W + 31u) / 32u;
+    const uint32_t b0 = nb * seg / nseg, b1 = seg < nseg ? nb * (seg + 1u) / nseg : b0;
+    for (uint32_t j0 = 0; j0 < N; j0 += 32u * UC) {
+        uint32_t a[UC];
 #pragma unroll
-        for (uint32_t q = 0; q < kUnits; ++q)
-            a[q] = 0u;
-        for (uint32_t w = warp; w * 32u < D; w += nw) {
-            uint32_t bits = gp[w];
-            while (bits) {
-                const uint32_t k = w * 32u + (uint32_t)(__ffs(bits) - 1);
-                bits &= bits - 1u;
+        for (int u = 0; u < UC; ++u)
+            a[u] = 0u;
+        for (uint32_t rho = id & 31u; rho < 32u; rho += workers) {
+            uint32_t win[16];
+            bool ready = false;   // win holds the words before this block
+            for (uint32_t b = b0; b < b1; ++b) {
+                const uint32_t w = 32u * b + lane;
+                const uint32_t bits = __ballot_sync(0xFFFFFFFFu, w < W && ((gp[w] >> rho) & 1u));
+                const uint32_t* y = S + j0 + rho + 1024u * b + lane;
+                if (j0 + rho + 1024u * b + 32u * (UC + 30u) + 31u < s_len) {
+                    if (!ready) {
 #pragma unroll
-                for (uint32_t q = 0; q < kUnits; ++q) {
-                    const uint32_t j = j0 + 32u * q + lane;
-                    if (q < uc && j < N)
-                        a[q] ^= S[k + j];
+                        for (int i = 0; i + 1 < UC; ++i)
+                            win[i] = y[32 * i];
+                        ready = true;
+                    }
+#pragma unroll 1
+                    for (uint32_t h = 0; h < 32u; h += 16u)
+                        jump_block16<UC>(bits >> h, y + 32u * h, a, win);
+                } else {
+                    for (uint32_t left = bits; left; left &= left - 1u) {
+                        const uint32_t k = (uint32_t)__ffs(left) - 1u;
+#pragma unroll
+                        for (int u = 0; u < UC; ++u)
+                            if (j0 + 32u * u + lane < N)
+                                a[u] ^= y[32u * k + 32u * u];
+                    }
                 }
             }
         }
 #pragma unroll
-        for (uint32_t q = 0; q < kUnits; ++q) {
-            const uint32_t j = j0 + 32u * q + lane;
-            if (q < uc && j < N && a[q])
-                atomicXor(&acc[j], a[q]);
+        for (int u = 0; u < UC; ++u) {
+            const uint32_t j = j0 + 32u * u + lane;
+            if (j < N && a[u])
+                atomicXor(&acc[j], a[u]);
         }
     }
-    __syncthreads();
+    if (parts > 1u) {
+        // the other parts' accumulators into part 0's, over the cluster's
+        // shared memory; every part has read the state row by now
+        cluster.sync();
+        if (part) {
+            uint32_t* sum = cluster.map_shared_rank(acc, 0);
+            for (uint32_t j = threadIdx.x; j < N; j += blockDim.x)
+                atomicXor(sum + j, acc[j]);
+        }
+        cluster.sync();
+        if (part)
+            return;
+    } else {
+        __syncthreads();
+    }
     // one ordinary step on the accumulated window: the state after J steps is
     // (acc[1] .. acc[N-1], new word), oldest first
     for (uint32_t j = threadIdx.x; j + 1u < N; j += blockDim.x)
@@ -475,6 +583,22 @@ __global__ void __launch_bounds__(256) mtgp_jump_kernel(const KParams P, uint32_
         y ^= acc[pos] >> sh2;
         g[N - 1u] = y ^ R[y & 15u];
     }
+}
+
+// The instantiation for N words: the units of one pass, N split into the
+// fewest passes of at most 12 units.
+const void* jump_fn(uint32_t N)
+{
+    const uint32_t U = (N + 31u) / 32u, passes = (U + 11u) / 12u, uc = (U + passes - 1u) / passes;
+    if (uc <= 4u)
+        return (const void*)mtgp_jump_kernel<4>;
+    if (uc == 5u)
+        return (const void*)mtgp_jump_kernel<5>;
+    if (uc <= 8u)
+        return (const void*)mtgp_jump_kernel<8>;
+    if (uc <= 10u)
+        return (const void*)mtgp_jump_kernel<10>;
+    return uc == 11u ? (const void*)mtgp_jump_kernel<11> : (const void*)mtgp_jump_kernel<12>;
 }
 
 // ---------------------------------------------------------------------------
@@ -805,10 +929,11 @@ mtgp_status mtgp::build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>
         if (e != cudaSuccess)
             return fail_cuda(e, "cudaMemcpy(parameter sets)");
     }
-    // distinct lengths per parameter set
+    // distinct lengths per parameter set (runs of one set and length, the
+    // usual case, are entered once)
     std::map<uint32_t, std::vector<uint64_t>> lengths;
     for (size_t i = 0; i < rows.size(); ++i)
-        if (jumps[i])
+        if (jumps[i] && !(i && jumps[i] == jumps[i - 1] && sets[i] == sets[i - 1]))
             lengths[sets[i]].push_back(jumps[i]);
     std::map<std::pair<uint32_t, uint64_t>, uint32_t> poly_index;
     std::vector<const Poly*> polys;
@@ -826,27 +951,32 @@ mtgp_status mtgp::build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>
         }
     }
     uint32_t max_deg = 0;
-    for (size_t i = 0; i < rows.size(); ++i) {
+    JumpItem ji{};
+    out->items.reserve(rows.size());
+    for (size_t i = 0, prev = 0; i < rows.size(); ++i) {
         if (!jumps[i])
             continue;
-        const uint32_t pi = poly_index.at(std::make_pair(sets[i], jumps[i]));
-        JumpItem ji;
+        if (out->items.empty() || jumps[i] != jumps[prev] || sets[i] != sets[prev]) {
+            ji.poly = poly_index.at(std::make_pair(sets[i], jumps[i]));
+            ji.deg = (uint32_t)std::max(degree(*polys[ji.poly]), 0);
+            ji.set = sets[i];
+            max_deg = std::max(max_deg, ji.deg);
+        }
+        prev = i;
         ji.stream = rows[i];
-        ji.poly = pi;
-        ji.deg = (uint32_t)std::max(degree(*polys[pi]), 0);
-        ji.set = sets[i];
         out->items.push_back(ji);
-        max_deg = std::max(max_deg, ji.deg);
     }
     if (out->items.empty())
         return MTGP_OK;
     const uint32_t N = st->P.k.n;
     out->words = (max_deg + 1 + 31) / 32;
     out->poly_words.assign(polys.size() * (size_t)out->words, 0u);
-    for (size_t i = 0; i < polys.size(); ++i)
-        for (int k = 0; k <= degree(*polys[i]); ++k)
-            if (bit(*polys[i], (size_t)k))
-                out->poly_words[i * out->words + (size_t)k / 32] |= 1u << (k % 32);
+    for (size_t i = 0; i < polys.size(); ++i) {
+        uint32_t* to = out->poly_words.data() + i * out->words;
+        const Poly& g = *polys[i];
+        for (uint32_t k = 0; k < out->words && k / 2u < g.size(); ++k)
+            to[k] = (uint32_t)(g[k / 2u] >> (32u * (k & 1u)));
+    }
     // a zero g (possible only if t^(J-1) = 0 mod mu, which needs t | mu):
     // the kernel then accumulates nothing and applies one step to 0
     out->smem = ((size_t)max_deg + 1 + N - 1 + N) * 4;
@@ -854,7 +984,14 @@ mtgp_status mtgp::build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess)
         return fail_cuda(e, "cudaGetDevice");
-    e = allow_max_dynamic_smem((const void*)mtgp_jump_kernel, dev, out->smem);
+    // with room behind the sequence for the last windows, unless only the
+    // sequence itself fits
+    const size_t room = 32u * (12u + 64u) * 4u;
+    e = allow_max_dynamic_smem(jump_fn(N), dev, out->smem + room);
+    if (e == cudaSuccess)
+        out->smem += room;
+    else if (e == cudaErrorInvalidValue)
+        e = allow_max_dynamic_smem(jump_fn(N), dev, out->smem);
     if (e == cudaErrorInvalidValue)
         return fail(MTGP_EINVAL, "state size too large for the jump kernel (%zu bytes of shared memory)",
                     out->smem);
@@ -869,8 +1006,28 @@ cudaError_t mtgp::launch_jump_batch(const mtgp_streams* st, uint32_t* rows_base,
 {
     if (n == 0)
         return cudaSuccess;
-    mtgp_jump_kernel<<<n, 256, smem, s>>>(st->P.k, rows_base, d_items, d_polys, words, st->d_sets);
-    return cudaGetLastError();
+    // Few jumps leave most of the chip idle, so each is shared out over a
+    // cluster of up to 8 CTAs, as long as every CTA still has an SM to itself.
+    uint32_t parts = 1;
+    while (parts < 8u && 2u * parts * n <= (uint32_t)st->sms)
+        parts *= 2u;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(n * parts);
+    c.blockDim = dim3(32u * kJumpWarps);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = parts;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    KParams P = st->P.k;
+    const KSet* sets = st->d_sets;
+    uint32_t s_len = (uint32_t)(smem / 4u) - P.n;
+    void* args[] = {&P, &rows_base, (void*)&d_items, (void*)&d_polys, &words, (void*)&sets, &s_len};
+    return cudaLaunchKernelExC(&c, jump_fn(P.n), args);
 }
 
 extern "C" mtgp_status mtgp_jump(mtgp_streams_t st, const uint32_t* ids, const uint64_t* jumps, uint32_t n,
@@ -880,15 +1037,32 @@ extern "C" mtgp_status mtgp_jump(mtgp_streams_t st, const uint32_t* ids, const u
         if (!st || (n && (!ids || !jumps)))
             return fail(MTGP_EINVAL, "null argument");
         DeviceGuard dg(st->device);
-        // total jump per stream (jumps compose additively)
-        std::map<uint32_t, uint64_t> total;
+        // total jump per stream (jumps compose additively), streams ascending
+        std::vector<std::pair<uint32_t, uint64_t>> total(n);
+        bool ascending = true;
         for (uint32_t i = 0; i < n; ++i) {
             if (ids[i] >= st->n_streams)
                 return fail(MTGP_EINVAL, "stream id %u out of range (%u streams)", ids[i], st->n_streams);
-            uint64_t& t = total[ids[i]];
-            if (t + jumps[i] < t)
-                return fail(MTGP_EINVAL, "total jump of stream %u overflows 64 bits", ids[i]);
-            t += jumps[i];
+            ascending = ascending && (i == 0 || ids[i] > ids[i - 1]);
+            total[i] = std::make_pair(ids[i], jumps[i]);
+        }
+        if (!ascending) {
+            std::stable_sort(total.begin(), total.end(),
+                             [](const std::pair<uint32_t, uint64_t>& a, const std::pair<uint32_t, uint64_t>& b) {
+                                 return a.first < b.first;
+                             });
+            size_t k = 0;
+            for (size_t i = 0; i < total.size(); ++i) {
+                if (k && total[k - 1].first == total[i].first) {
+                    uint64_t& t = total[k - 1].second;
+                    if (t + total[i].second < t)
+                        return fail(MTGP_EINVAL, "total jump of stream %u overflows 64 bits", total[i].first);
+                    t += total[i].second;
+                } else {
+                    total[k++] = total[i];
+                }
+            }
+            total.resize(k);
         }
         // set index of each stream (per-stream parameter sets)
         std::vector<uint32_t> set_of_stream;
@@ -899,6 +1073,9 @@ extern "C" mtgp_status mtgp_jump(mtgp_streams_t st, const uint32_t* ids, const u
         }
         std::vector<uint32_t> rows, sets;
         std::vector<uint64_t> lens;
+        rows.reserve(total.size());
+        sets.reserve(total.size());
+        lens.reserve(total.size());
         for (const auto& kv : total) {
             rows.push_back(kv.first);
             sets.push_back(st->d_sets ? set_of_stream[kv.first] : 0u);
@@ -911,27 +1088,23 @@ extern "C" mtgp_status mtgp_jump(mtgp_streams_t st, const uint32_t* ids, const u
         if (b.items.empty())
             return ok();
         cudaStream_t cs = (cudaStream_t)cuda_stream;
-        void *d_items = nullptr, *d_polys = nullptr;
-        J_TRY(cudaMallocAsync(&d_items, b.items.size() * sizeof(JumpItem), cs), "cudaMallocAsync");
-        cudaError_t e = cudaMallocAsync(&d_polys, b.poly_words.size() * 4, cs);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(d_items, b.items.data(), b.items.size() * sizeof(JumpItem),
-                                cudaMemcpyHostToDevice, cs);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(d_polys, b.poly_words.data(), b.poly_words.size() * 4,
-                                cudaMemcpyHostToDevice, cs);
-        if (e == cudaSuccess)
-            e = launch_jump_batch(st, st->d_states, (const JumpItem*)d_items, (uint32_t)b.items.size(),
-                                  (const uint32_t*)d_polys, b.words, b.smem, cs);
-        // the host arrays above are locals: wait for the copies before returning
-        const cudaError_t e2 = cudaStreamSynchronize(cs);
-        if (d_polys)
-            cudaFreeAsync(d_polys, cs);
-        cudaFreeAsync(d_items, cs);
-        if (e != cudaSuccess)
-            return fail_cuda(e, "jump kernel");
-        if (e2 != cudaSuccess)
-            return fail_cuda(e2, "cudaStreamSynchronize");
+        // items and polynomials go up in one copy from a pinned slot of the
+        // handle's ring (no allocation per call)
+        TableSlot& sl = st->slots[st->next_slot];
+        st->next_slot = (st->next_slot + 1) % (int)st->slots.size();
+        const size_t b_items = b.items.size() * sizeof(JumpItem), o_poly = (b_items + 15u) & ~(size_t)15u;
+        const size_t bytes = o_poly + b.poly_words.size() * 4u;
+        r = reserve_slot(sl, bytes);
+        if (r != MTGP_OK)
+            return r;
+        std::memcpy(sl.host, b.items.data(), b_items);
+        std::memcpy((char*)sl.host + o_poly, b.poly_words.data(), b.poly_words.size() * 4u);
+        J_TRY(cudaMemcpyAsync(sl.dev, sl.host, bytes, cudaMemcpyHostToDevice, cs), "cudaMemcpyAsync(jumps)");
+        J_TRY(launch_jump_batch(st, st->d_states, (const JumpItem*)sl.dev, (uint32_t)b.items.size(),
+                                (const uint32_t*)((char*)sl.dev + o_poly), b.words, b.smem, cs), "jump kernel");
+        J_TRY(cudaEventRecord(sl.ev, cs), "cudaEventRecord");
+        sl.ev_recorded = true;
+        J_TRY(cudaStreamSynchronize(cs), "cudaStreamSynchronize");
         return ok();
     } catch (const std::bad_alloc&) {
         return fail(MTGP_ENOMEM, "host allocation failed");
