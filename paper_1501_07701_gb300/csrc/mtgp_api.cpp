@@ -729,6 +729,11 @@ LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_
         // whose three busy warps may share a quarter, 0.53 apart)
         c.warps_per_cta = 4;
         c.ctas_per_sm = 1;
+    } else if (st->P.k.n < 257u && total / std::max<uint64_t>(max_item, 1) >= 16u * sms) {
+        // short states have the latency of a 32-column step to hide (4096 x
+        // 2^18 at Mexp 3217: 1.05 ms at 16 warps, 1.14 at 12, 1.40 at 8)
+        c.warps_per_cta = 8;
+        c.ctas_per_sm = 2;
     } else if (total / std::max<uint64_t>(max_item, 1) >= 12u * sms ||
                (n_items > 8u * sms && max_item * n_items <= total + total / 8u)) {
         // 12 warps per SM run 1-2 % faster than 8 and end evenly, when no

@@ -432,16 +432,104 @@ __device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const R
     });
 }
 
+// nfull consecutive full rows of one request for short states (M < 9, no
+// 128-word step fits): the same late tempering and wrapped addresses, one
+// 32-column sub-step at a time, each with the next sub-step's words read
+// before its own are written.  That is exact while N - pos >= 64: none of
+// those words is written by the current sub-step, and a wrapped pick-up lands
+// on a column of an earlier, already written sub-step.
+// What bounds it: the chain of a sub-step (lookup, store, barrier) at few
+// warps, the LSU and ALU at many; 101 of 128 lanes work at Mexp 3217.
+// Measured there against steps of 64 words read, passed and written: uneven
+// workload unsplit 9.9 -> 5.6 ms, split in pieces of 701 932 6.4 -> 4.7 ms,
+// 2432 equal streams at 16 warps per SM 721 -> 1098 Gnumbers/s.
+template <int M, int FMT>
+__device__ __forceinline__ void gen_rows_short(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
+                                               const uint32_t* __restrict__ Tb, uint32_t nfull)
+{
+    static_assert(M >= 3 && M <= 8, "two packed index registers, and a neighbour of column N-1 in time");
+    constexpr int TT = FMT == 0 ? 64 : 128;
+    constexpr int NT = (M + 3) / 4;
+    const uint32_t N = P.n, last_lane = (N - 1u) & 31u;
+    uint32_t sa = saddr(S + lane);
+    uint32_t x1_last = lane >= last_lane ? saddr(S) : sa + 128u * (M - 1) + 4u;
+    uint32_t tb = saddr(Tb);
+    uint32_t mul1 = 1u << P.sh1;   // on the FMA pipe, as in gen_rows_late
+    asm volatile("" : "+r"(mul1), "+r"(sa), "+r"(x1_last), "+r"(tb));
+    uint32_t r[M], qa[M], T[NT], xs[4 * NT];
+    static_for<M>([&](auto im) {
+        constexpr int m = im.value;
+        const uint32_t p = 32u * m + lane + P.pos;
+        r[m] = lds_at<128 * m>(sa);
+        qa[m] = saddr(S + (p < N ? p : p - N));
+        asm volatile("" : "+r"(qa[m]));
+    });
+    static_for<NT>([&](auto i) { T[i.value] = 0u; });
+    static_for<4 * NT>([&](auto i) { xs[i.value] = 0u; });
+    T[NT - 1] = (temper_index(S[P.pos - 1u]) & 15u) << (2 + 8 * ((M - 1) & 3));
+    uint32_t x1 = lds_at<4>(sa), xp = lds_at<0>(qa[0]);
+    uint32_t* op = ow + 1 - (int)N;
+#pragma unroll 4
+    for (uint32_t q = 0; q < nfull; ++q, op += N) {
+        const bool body = q != 0u;
+        const bool last = lane == last_lane || (body && lane < last_lane);
+        static_for<M>([&](auto im) {
+            constexpr int m = im.value, n = m + 1 < M ? m + 1 : 0;
+            uint32_t y1;
+            if constexpr (n + 1 < M)
+                y1 = lds_at<128 * n + 4>(sa);
+            else
+                y1 = lds_at<0>(x1_last);
+            const uint32_t yp = lds_at<0>(qa[n]);
+            const uint32_t yy = (r[m] & P.mask) ^ x1;
+            const uint32_t y = yy ^ (yy * mul1) ^ (xp >> P.sh2);
+            r[m] = y ^ tbl(Tb, 0u, y);
+            const uint32_t tw = lds_at<TT>(__byte_perm(T[m / 4], tb, 0x7650 + m % 4));
+            const uint32_t o = finish<FMT>(x1, tw);
+            xs[m] = xp;
+            sts_at<128 * m>(sa, r[m]);
+            if (m + 1 < M ? body : last)
+                __stcs(op + 32 * m, o);
+            __syncwarp();
+            x1 = y1;
+            xp = yp;
+        });
+        static_for<NT>([&](auto i) {
+            constexpr int b = 4 * i.value;
+            const uint32_t x4[4] = {xs[b], xs[b + 1], xs[b + 2], xs[b + 3]};
+            T[i.value] = temper_pack(x4);
+        });
+    }
+    static_for<M>([&](auto im) {
+        constexpr int m = im.value;
+        const uint32_t v = lds_at<128 * m + 4>(sa);
+        const uint32_t tw = lds_at<TT>(__byte_perm(T[m / 4], tb, 0x7650 + m % 4));
+        if (m + 1 < M || lane < last_lane)
+            __stcs(op + 32 * m, finish<FMT>(v, tw));
+    });
+}
+
+template <int M, int FMT>
+__device__ __forceinline__ void gen_full_rows(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
+                                              const uint32_t* __restrict__ Tb, uint32_t nfull)
+{
+    if constexpr (M < 9)
+        gen_rows_short<M, FMT>(S, ow, P, lane, Tb, nfull);
+    else
+        gen_rows_late<M, FMT>(S, ow, P, lane, Tb, nfull);
+}
+
 // A row on the same layout (no mirror) with its numbers stored at once:
-// columns 0 .. n_valid-1.  SLOW: the row crosses into another request and
-// every lane finds its own; otherwise the row's numbers go to `ow`.
+// columns 0 .. n_valid-1, in steps of 128 words, 64 for short states.  SLOW:
+// the row crosses into another request and every lane finds its own;
+// otherwise the row's numbers go to `ow`.
 template <int M, int FMT, bool SLOW>
 __device__ __forceinline__ void gen_row_part(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
                                              const uint32_t* __restrict__ Tb, uint32_t n_valid,
                                              uint64_t row_g, const Segment* __restrict__ segs,
                                              uint32_t s_first, uint32_t s_end, uint32_t* __restrict__ out)
 {
-    constexpr int K = 4;
+    constexpr int K = M < 9 ? 2 : 4;
     const uint32_t N = P.n;
     uint32_t* const Sw = S + lane;
 #pragma unroll 1
@@ -476,8 +564,8 @@ __device__ __forceinline__ void gen_row_part(uint32_t* S, uint32_t* ow, const Ro
     }
 }
 
-// Advances one stream whose N - pos >= 256 by the segments [s_begin, s_end),
-// this warp alone.
+// Advances one stream whose N - pos >= 256 (>= 64 for short states) by the
+// segments [s_begin, s_end), this warp alone.
 template <int M>
 __device__ __forceinline__ void run_item_late(const KParams& KP, const RowP& P, uint32_t* __restrict__ g,
                                               uint32_t* __restrict__ S, const Segment* __restrict__ segs,
@@ -505,11 +593,11 @@ __device__ __forceinline__ void run_item_late(const KParams& KP, const RowP& P, 
             // the rows that lie wholly inside this request, back to back
             const uint32_t nfull = (uint32_t)min((seg_end - row) / N, (uint64_t)0xFFFFFFFFu);
             if (sg.fmt == 0)
-                gen_rows_late<M, 0>(S, ow, P, lane, Tb, nfull);
+                gen_full_rows<M, 0>(S, ow, P, lane, Tb, nfull);
             else if (sg.fmt == 1)
-                gen_rows_late<M, 1>(S, ow, P, lane, Tb, nfull);
+                gen_full_rows<M, 1>(S, ow, P, lane, Tb, nfull);
             else
-                gen_rows_late<M, 2>(S, ow, P, lane, Tb, nfull);
+                gen_full_rows<M, 2>(S, ow, P, lane, Tb, nfull);
             row += (uint64_t)nfull * N;
         } else {
             const uint64_t left = total - row;
@@ -632,21 +720,25 @@ __device__ __forceinline__ void run_item(const KParams& KP, const RowP& P, uint3
         __syncwarp();
 }
 
-// One stream on one warp: the late-tempering loop where its 128-word steps
-// fit (N - pos >= 256), else the general one.
+// One stream on one warp: the late-tempering loops where their steps fit
+// (N - pos >= 256, short states always), else the general one.
 template <int M, int K>
 __device__ __forceinline__ void run_single(const KParams& KP, const RowP& P, uint32_t* __restrict__ g,
                                            uint32_t* __restrict__ S, const Segment* __restrict__ segs,
                                            uint32_t s_begin, uint32_t s_end, uint32_t* __restrict__ out,
                                            uint32_t warp, uint32_t lane, const uint32_t* __restrict__ Tb)
 {
-    if constexpr (K == 4 && M >= 9) {
+    if constexpr (M < 9) {   // 32 K <= N - pos, so N - pos >= 64
+        run_item_late<M>(KP, P, g, S, segs, s_begin, s_end, out, lane, Tb);
+        return;
+    } else if constexpr (K == 4) {
         if (P.n - P.pos >= 256u) {
             run_item_late<M>(KP, P, g, S, segs, s_begin, s_end, out, lane, Tb);
             return;
         }
     }
-    run_item<M, K, 1>(KP, P, g, S, segs, s_begin, s_end, out, warp, lane, Tb);
+    if constexpr (M >= 9)
+        run_item<M, K, 1>(KP, P, g, S, segs, s_begin, s_end, out, warp, lane, Tb);
 }
 
 // Claims.  The n items (longest first) are dealt to n_groups lists, one per
@@ -726,11 +818,12 @@ __device__ __forceinline__ uint32_t claim_item(Claims& c, uint32_t lane)
 // smaller states (168 registers), 8 for the larger ones, which keep three
 // words per column group.  At 16 warps (128 registers) the late loop spilled
 // and ran at 1190 instead of 1400 Gnumbers/s (2432 equal streams, Mexp 11213).
-// The other row loops need few registers and gain from many warps: 16 per SM,
-// 32 for short states.
+// Short states, with a chain of 32-column sub-steps to hide, run best at 16
+// (2432 equal streams at Mexp 3217: 1098 Gnumbers/s; at 24 and 32 warps per SM
+// the loop spills and runs at 840); the other row loops need few registers.
 constexpr int fast_min_ctas(int M, int K, int G)
 {
-    return (M < 9 ? 32 : K != 4 ? 16 : M < 16 ? 12 : 8) / G;
+    return (M < 9 || K != 4 ? 16 : M < 16 ? 12 : 8) / G;
 }
 
 // Persistent kernel.  Phase 1: the CTA claims the longest streams (items

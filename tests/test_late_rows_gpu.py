@@ -1,4 +1,4 @@
-"""The late-tempering row loop (N - pos >= 256) and the per-SM claim lists:
+"""The late-tempering row loops (N - pos >= 256, and short states) and the per-SM claim lists:
 every output and state against the oracle, tolerance zero, at the sizes where
 they can go wrong: counts one off whole rows and whole passes of the unrolled
 loop, requests that start and end inside rows, few items, and more items than
@@ -37,7 +37,7 @@ def _check(mexp, ids, counts, fmt, n_streams, cfg=None, calls=2):
 
 
 @pytest.mark.parametrize("fmt", [0, 1, 2])
-@pytest.mark.parametrize("mexp", [9689, 11213, 19937, 23209, 44497])
+@pytest.mark.parametrize("mexp", [3217, 4253, 4423, 9689, 11213, 19937, 23209, 44497])
 def test_counts_around_whole_rows(mexp, fmt):
     n = mexp // 32 + 1
     rows = [0, 1, 2, 3, 4, 5, 8, 9]
@@ -45,7 +45,7 @@ def test_counts_around_whole_rows(mexp, fmt):
     _check(mexp, np.arange(len(counts)), counts, fmt, len(counts))
 
 
-@pytest.mark.parametrize("mexp", [11213, 44497])
+@pytest.mark.parametrize("mexp", [3217, 11213, 44497])
 def test_requests_that_meet_inside_rows(mexp):
     n = mexp // 32 + 1
     rng = np.random.default_rng(mexp)
