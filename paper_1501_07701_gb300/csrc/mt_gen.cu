@@ -12,7 +12,7 @@
 // so a step needs one __syncwarp, at its end.  When the window reaches the end
 // of the buffer, its n live words are moved back to the start.
 //
-// Per number: three shared loads, one shared store, one coalesced global
+// Per number: two or three shared loads, one shared store, one coalesced global
 // store.  The twist and the tempering are register arithmetic; the two left
 // shifts of the tempering run as integer multiplies on the FMA pipe.
 #include <algorithm>
@@ -81,6 +81,35 @@ __device__ __forceinline__ uint32_t mt_convert_rt(uint32_t z, uint32_t fmt)
     return fmt == 0 ? z : (fmt == 1 ? mt_convert<1>(z) : mt_convert<2>(z));
 }
 
+__device__ __forceinline__ uint32_t mt_lds(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void mt_sts(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+template <int K, int FMT>
+__device__ __forceinline__ void mt_run_steps(const MtK& P, const MtSet& S, uint32_t* bp, uint32_t* op,
+                                             uint32_t nst, uint32_t lane);
+
+// Whole steps, by the loop that fits the set.
+template <int K, int FMT>
+__device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32_t* buf, uint32_t* op,
+                                            uint32_t nst, uint32_t lane);
+template <int K, int FMT>
+__device__ __forceinline__ void mt_run(const MtK& P, const MtSet& S, uint32_t* bp, uint32_t* op, uint32_t nst,
+                                       uint32_t lane)
+{
+    if (S.W == P.n - S.m)
+        mt_run_wide<K, FMT>(P, S, bp, op, nst, lane);
+    else
+        mt_run_steps<K, FMT>(P, S, bp, op, nst, lane);
+}
+
 // `nst` >= 1 whole steps inside one request, with room in the buffer for all
 // of them.  Lane j of sub-step i takes number k0 + 32 i + j of each step;
 // bp = buf + off + lane and op = the lane's output of the first step.
@@ -135,6 +164,72 @@ __device__ __forceinline__ void mt_run_steps(const MtK& P, const MtSet& S, uint3
         if (act[i])
             __stcs(op + 32 * i, o);
     }
+}
+
+// The same for sets whose step is as wide as the recurrence allows, W = n - m
+// (n - m <= 256: the seed-generated sets up to n = 512, MT19937).
+//
+// The middle word x_{k+W+m} of the next step's number is then the word x_{k+n}
+// that the same lane has just made, so it stays in a register: two shared
+// loads per number instead of three, and they fly while the step's numbers
+// are tempered, converted and stored.  The chain from step to step is twist,
+// store, barrier and load.  Lanes past W store too, behind the step's words
+// (in the buffer's slack at its end): only words of later steps come there,
+// each stored before it is read.
+// What bounds it: that chain, 130 cycles per step for a warp alone and 172 for
+// two warps per SM quarter (p = 3217, 51 numbers per step).  Measured: the
+// uneven 10 000-stream workload 7.80 -> 6.85 ms at p = 3217 and 6.94 -> 6.06 ms
+// for MT19937.  Reading a whole step ahead, with the one or two words it then
+// lacks at p = 3217 by shuffle, took more instructions than it hid latency
+// (9.6 ms).
+template <int K, int FMT>
+__device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32_t* buf, uint32_t* op,
+                                            uint32_t nst, uint32_t lane)
+{
+    const uint32_t W = S.W, upper = P.upper;
+    const uint32_t step = 4u * W;
+    uint32_t rd = (uint32_t)__cvta_generic_to_shared(buf);   // this lane's x_k
+    uint32_t wr = rd + 4u * P.n;                             // and x_{k+n}
+    bool act[K];
+    uint32_t x0[K], x1[K], xm[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        act[i] = 32u * i + lane < W;
+        x0[i] = mt_lds(rd + 128u * i);
+        x1[i] = mt_lds(rd + 128u * i + 4u);
+        xm[i] = mt_lds(rd + 128u * i + 4u * S.m);
+    }
+    constexpr int U = K == 4 ? 4 : 2;   // as measured per step width
+#pragma unroll U
+    for (uint32_t t = 0; t < nst; ++t) {
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            xm[i] = mt_twist(upper, S, x0[i], x1[i], xm[i]);
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            mt_sts(wr + 128u * i, xm[i]);
+        __syncwarp();
+        rd += step;
+        wr += step;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            x0[i] = mt_lds(rd + 128u * i);
+            x1[i] = mt_lds(rd + 128u * i + 4u);
+        }
+        uint32_t o[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            o[i] = mt_convert<FMT>(mt_temper(S, xm[i]));
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            asm volatile("" : "+r"(o[i]));   // not moved under the store's condition
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            if (act[i])
+                __stcs(op + 32 * i, o[i]);
+        op += W;
+    }
+    __syncwarp();   // the loads above come before the buffer's next writes
 }
 
 // A step that crosses a request boundary or the stream's end: each lane finds
@@ -234,11 +329,11 @@ __global__ void __launch_bounds__(128) mt_gen_kernel(const MtK P, uint32_t* __re
                 const uint32_t nst = n_seg < n_buf ? (uint32_t)n_seg : n_buf;
                 uint32_t* op = out + (sg.out_off - sg.g_start) + k0 + lane;
                 if (sg.fmt == 0)
-                    mt_run_steps<K, 0>(P, S, bp, op, nst, lane);
+                    mt_run<K, 0>(P, S, bp, op, nst, lane);
                 else if (sg.fmt == 1)
-                    mt_run_steps<K, 1>(P, S, bp, op, nst, lane);
+                    mt_run<K, 1>(P, S, bp, op, nst, lane);
                 else
-                    mt_run_steps<K, 2>(P, S, bp, op, nst, lane);
+                    mt_run<K, 2>(P, S, bp, op, nst, lane);
                 k0 += (uint64_t)nst * W;
                 off += nst * W;
             } else {
@@ -616,7 +711,10 @@ extern "C" mtgp_status mtgp_mt_generate(mtgp_mt_t h, const uint32_t* ids, const 
         const uint32_t n_items = (uint32_t)w.items.size();
         const long long pace = (long long)((w.total + w.max_item - 1) / w.max_item);
         const long long warps = std::max<long long>(pace, (long long)h->sms * kWarpsPerCta);
-        const long long want = (std::min<long long>(n_items, warps) + kWarpsPerCta - 1) / kWarpsPerCta;
+        long long want = (std::min<long long>(n_items, warps) + kWarpsPerCta - 1) / kWarpsPerCta;
+        // a few CTAs over a whole number per SM would slow those SMs' streams
+        if (want > h->sms && want % h->sms <= h->sms / 8)
+            want -= want % h->sms;
         const int grid = (int)std::max(1LL, std::min<long long>(want, h->grid_cap));
         const WorkItem* items = (const WorkItem*)((char*)sl.dev + io);
         const Segment* segs = (const Segment*)((char*)sl.dev + so);
