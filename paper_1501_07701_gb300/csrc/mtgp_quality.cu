@@ -43,18 +43,60 @@ struct GapEdge {
 // c of the launch is found from the prefix sums of those chunk counts.  Warps
 // claim runs of `run` consecutive chunks from an atomic counter, so a warp's
 // consecutive chunks mostly share a sequence and its histogram, which is
-// flushed to global memory only when the sequence changes.  Per group of 32
-// consecutive values the visits form a ballot mask B; a visiting lane's gap
-// is the distance to the nearest lower visiting lane, or the carried run D
-// plus its lane index if it is the group's first visit (the first visit of a
-// chunk is left to the stitch kernel); both cases are one expression,
-// gap = lane - 1 - prev with prev = -1 - D when no lower lane visits.  Loads
-// run a round ahead of the scan: the kG groups of the next round are in
-// flight while the current round is scanned, and rounds with every value
-// present are scanned without per-lane bounds checks.  The ballot and every
-// shuffle run in warp-uniform control flow; the per-lane branch holds only
-// shared-memory atomics.
-constexpr uint32_t kG = 8;      // groups of 32 values per load round
+// flushed to global memory only when the sequence changes.
+//
+// A chunk is scanned in rounds of 32 groups of 32 consecutive values.  Each
+// group's visits form a ballot, and lane g keeps the ballot of group g; so a
+// value costs its load, its test and a share of a vote.  After the round
+// every lane holds 32 consecutive values' visits as one word: it finds the
+// visit before its first one (the highest lower lane with a visit, or the
+// carried run D) and walks its set bits, counting one gap each in shared
+// memory.  The first visit of a chunk is left to the stitch kernel.  Loads run
+// a batch of kG groups ahead of the tests.  All of it is warp-uniform control
+// flow: a loop that each lane left when its word was used up ran its lanes one
+// by one (3.45 ms for 2^30 values).
+// What bounds it: HBM reads (2^30 values in 0.65 ms, 6.6 TB/s, 97 % of the
+// copy rate).  The first version resolved every group's gaps by itself, with a
+// dependent chain per 32 values: 65 %.
+constexpr uint32_t kG = 8;      // groups of 32 values per load batch
+
+// Visits of a round: word w of lane g = the ballot of group g (values 32 g ..
+// 32 g + 31 of the round, nv values in all).  Counts their gaps; D, P and seen
+// are the chunk's carried run, the run before its first visit and whether it
+// had one.
+__device__ __forceinline__ void gap_round(uint32_t w, uint32_t nv, uint32_t lane, uint32_t lower, uint32_t* h,
+                                          uint32_t t, uint32_t& D, uint32_t& P, bool& seen)
+{
+    const uint32_t nz = __ballot_sync(0xFFFFFFFFu, w != 0u);
+    if (!nz) {
+        D += nv;
+        return;
+    }
+    const int last = (int)(32u * lane) + 31 - __clz(w);   // this lane's last visit (if it has one)
+    const uint32_t below = nz & lower;
+    const int pv = __shfl_sync(0xFFFFFFFFu, last, below ? 31 - __clz(below) : 0);
+    int prev = below ? pv : -1 - (int)D;
+    if (!seen) {
+        const int fl = __ffs(nz) - 1;
+        P = D + (uint32_t)__shfl_sync(0xFFFFFFFFu, (int)(32u * lane) + __ffs(w) - 1, fl);
+        if (!below && w) {   // this lane's first visit is the chunk's: not counted here
+            prev = (int)(32u * lane) + __ffs(w) - 1;
+            w &= w - 1u;
+        }
+        seen = true;
+    }
+    D = nv - 1u - (uint32_t)__shfl_sync(0xFFFFFFFFu, last, 31 - __clz(nz));
+    // one visit per lane and pass; lanes without one count in a slot of their
+    // own behind the histogram, so that a pass has no branch
+    const uint32_t hs = (uint32_t)__cvta_generic_to_shared(h), own = hs + 4u * (t + 1u + lane);
+    while (__any_sync(0xFFFFFFFFu, w != 0u)) {
+        const int at = (int)(32u * lane) + __ffs(w) - 1;
+        const uint32_t a = w ? hs + 4u * min((uint32_t)(at - prev - 1), t) : own;
+        asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory");
+        w &= w - 1u;
+        prev = at;
+    }
+}
 
 __device__ __forceinline__ void gap_flush(uint32_t* h, uint32_t t, unsigned long long* hs, uint32_t lane)
 {
@@ -92,11 +134,11 @@ __global__ void __launch_bounds__(kWarps * 32) mtgp_gap_kernel(const uint32_t* _
                                                               unsigned long long* __restrict__ hist,
                                                               GapEdge* __restrict__ edges)
 {
-    extern __shared__ uint32_t h_all[];   // kWarps histograms of t + 1 counts
+    extern __shared__ uint32_t h_all[];   // kWarps histograms of t + 1 counts and 32 slots
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t lower = (1u << lane) - 1u;   // lanes below this one
-    uint32_t* h = h_all + warp * (t + 1u);
-    for (uint32_t i = lane; i <= t; i += 32u)
+    uint32_t* h = h_all + warp * (t + 33u);
+    for (uint32_t i = lane; i < t + 33u; i += 32u)
         h[i] = 0u;
     __syncwarp();
     uint32_t cur = 0xFFFFFFFFu;
@@ -123,50 +165,59 @@ __global__ void __launch_bounds__(kWarps * 32) mtgp_gap_kernel(const uint32_t* _
             const uint32_t* v = values + seq_start[seq] + off;
             uint32_t D = 0, P = 0;
             bool seen = false;
-            uint32_t xa[kG];
-#pragma unroll
-            for (uint32_t g = 0; g < kG; ++g) {
-                const uint32_t idx = 32u * g + lane;
-                xa[g] = idx < len ? __ldcs(v + idx) : 0u;
-            }
-            // scans one round; `full`: all 32 kG values are present (no per-lane checks)
-            auto scan = [&](const uint32_t (&x)[kG], uint32_t base0, bool full) {
-#pragma unroll
-                for (uint32_t g = 0; g < kG; ++g) {
-                    const uint32_t base = base0 + 32u * g;
-                    if (!full && base >= len)
-                        break;
-                    const bool in = (x[g] & fmask) == 0u && (full || base + lane < len);
-                    const uint32_t B = __ballot_sync(0xFFFFFFFFu, in);
-                    const uint32_t below = B & lower;
-                    // position of the previous visit (-1 - D: D non-visits before this group)
-                    const int prev = below ? 31 - __clz(below) : -1 - (int)D;
-                    if (in && (below || seen))
-                        atomicAdd(&h[min((uint32_t)((int)lane - 1 - prev), t)], 1u);
-                    const uint32_t nv = full ? 32u : min(32u, len - base);
-                    const uint32_t hiB = 31u - __clz(B);
-                    P = (!seen && B) ? D + (uint32_t)(__ffs(B) - 1) : P;
-                    seen = seen || B;
-                    D = B ? nv - 1u - hiB : D + nv;
-                }
-            };
-            const uint32_t nfull = len / (32u * kG);   // rounds with every value present
-            uint32_t base0 = 0;
-            for (uint32_t q = 0; q < nfull; ++q, base0 += 32u * kG) {
-                uint32_t xb[kG];
-                const bool next_full = q + 1u < nfull;
-#pragma unroll
-                for (uint32_t g = 0; g < kG; ++g) {
-                    const uint32_t idx = base0 + 32u * (kG + g) + lane;
-                    xb[g] = (next_full || idx < len) ? __ldcs(v + idx) : 0u;
-                }
-                scan(xa, base0, true);
+            const uint32_t nfull = len / 1024u;   // rounds with every value present
+            uint32_t xa[kG], xb[kG];
+            if (nfull) {
 #pragma unroll
                 for (uint32_t g = 0; g < kG; ++g)
-                    xa[g] = xb[g];
+                    xa[g] = __ldcs(v + 32u * g + lane);
             }
-            if (base0 < len)
-                scan(xa, base0, false);
+            for (uint32_t q = 0; q < nfull; ++q) {
+                uint32_t w = 0;
+#pragma unroll
+                for (uint32_t b = 0; b < 32u; b += 2u * kG) {
+                    // batches b and b + kG of the round; each is loaded a batch ahead
+#pragma unroll
+                    for (uint32_t g = 0; g < kG; ++g)
+                        xb[g] = __ldcs(v + 1024u * q + 32u * (b + kG + g) + lane);
+#pragma unroll
+                    for (uint32_t g = 0; g < kG; ++g) {
+                        const uint32_t B = __ballot_sync(0xFFFFFFFFu, (xa[g] & fmask) == 0u);
+                        w = lane == b + g ? B : w;
+                    }
+                    if (b + 2u * kG < 32u || q + 1u < nfull) {
+#pragma unroll
+                        for (uint32_t g = 0; g < kG; ++g)
+                            xa[g] = __ldcs(v + 1024u * q + 32u * (b + 2u * kG + g) + lane);
+                    }
+#pragma unroll
+                    for (uint32_t g = 0; g < kG; ++g) {
+                        const uint32_t B = __ballot_sync(0xFFFFFFFFu, (xb[g] & fmask) == 0u);
+                        w = lane == b + kG + g ? B : w;
+                    }
+                }
+                gap_round(w, 1024u, lane, lower, h, t, D, P, seen);
+            }
+            if (1024u * nfull < len) {
+                uint32_t w = 0;
+#pragma unroll
+                for (uint32_t b = 0; b < 32u; b += kG) {
+                    if (1024u * nfull + 32u * b < len) {
+#pragma unroll
+                        for (uint32_t g = 0; g < kG; ++g) {
+                            const uint32_t idx = 1024u * nfull + 32u * (b + g) + lane;
+                            xa[g] = idx < len ? __ldcs(v + idx) : 0xFFFFFFFFu;
+                        }
+#pragma unroll
+                        for (uint32_t g = 0; g < kG; ++g) {
+                            const uint32_t idx = 1024u * nfull + 32u * (b + g) + lane;
+                            const uint32_t B = __ballot_sync(0xFFFFFFFFu, idx < len && (xa[g] & fmask) == 0u);
+                            w = lane == b + g ? B : w;
+                        }
+                    }
+                }
+                gap_round(w, len - 1024u * nfull, lane, lower, h, t, D, P, seen);
+            }
             if (lane == 0) {
                 GapEdge e;
                 e.prefix = seen ? P : len;
@@ -205,16 +256,21 @@ __global__ void __launch_bounds__(256) mtgp_gap_stitch_kernel(const uint64_t* __
 }
 
 // One warp per pair of blocks (2K values, K = L / s).  Each lane sums the
-// field weights of its values of each block; two warp reductions give the
-// block weights; lane 0 classifies them and counts the pair in the warp's
-// table, which is flushed whenever the warp moves to another sequence.
+// field weights of its values of each block; one warp reduction of both sums
+// packed into a word (two where L >= 2^16) gives the block weights; lane 0
+// classifies them and counts the pair in the warp's table, which is flushed
+// whenever the warp moves to another sequence.  A pair of up to 32 kB values
+// is loaded in one batch while the previous pair is reduced and counted.
+// What bounds it: HBM reads (2^30 values in 0.77 ms, 5.6 TB/s, 82 % of the copy
+// rate; the first version, with no loads in flight during its ten shuffles
+// and its counting, 68 %).
 __global__ void __launch_bounds__(kWarps * 32) mtgp_hamming_kernel(const uint32_t* __restrict__ values,
                                                                   const uint64_t* __restrict__ seq_start,
                                                                   const uint64_t* __restrict__ pair_base,
                                                                   uint32_t n_seq, uint64_t n_pairs,
                                                                   uint32_t fmask, uint32_t K,
                                                                   const uint32_t* __restrict__ bounds,
-                                                                  uint32_t n_bounds,
+                                                                  uint32_t n_bounds, bool packed,
                                                                   unsigned long long* __restrict__ table)
 {
     __shared__ uint32_t tab_all[kWarps][kMaxClasses * kMaxClasses];
@@ -232,11 +288,40 @@ __global__ void __launch_bounds__(kWarps * 32) mtgp_hamming_kernel(const uint32_
     const uint64_t gwarp = (uint64_t)blockIdx.x * kWarps + warp;
     const uint64_t per = (n_pairs + nwarps - 1) / nwarps;
     const uint64_t p0 = gwarp * per, p1 = min(p0 + per, n_pairs);
-    uint32_t seq = 0xFFFFFFFFu;
-    uint64_t seq_end = 0;
+    constexpr uint32_t kB = 16;   // values per lane and batch, all in flight
+    const bool one = 2u * K <= 32u * kB;   // the whole pair is one batch
+    uint32_t seq = 0xFFFFFFFFu;   // sequence of the counted pairs
     bool dirty = false;
+    uint32_t lseq = 0;            // sequence of the next pair to load
+    uint64_t lend = 0;
+    const uint32_t* lv = nullptr;
+    uint32_t xs[kB];
+    // finds pair p and loads its first batch
+    auto load = [&](uint64_t p) {
+        if (p >= lend) {
+            // the sequence holding pair p: last s with pair_base[s] <= p
+            uint32_t lo = 0, hi = n_seq;
+            while (hi - lo > 1u) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (pair_base[mid] <= p)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            lseq = lo;
+            lend = pair_base[lo + 1];
+        }
+        lv = values + seq_start[lseq] + (p - pair_base[lseq]) * 2ull * K;
+#pragma unroll
+        for (uint32_t q = 0; q < kB; ++q) {
+            const uint32_t j = 32u * q + lane;
+            xs[q] = j < 2u * K ? __ldcs(lv + j) : 0u;
+        }
+    };
+    if (p0 < p1)
+        load(p0);
     for (uint64_t p = p0; p < p1; ++p) {
-        if (seq == 0xFFFFFFFFu || p >= seq_end) {
+        if (seq != lseq) {
             if (dirty) {
                 __syncwarp();
                 for (uint32_t i = lane; i < C * C; i += 32u) {
@@ -247,43 +332,37 @@ __global__ void __launch_bounds__(kWarps * 32) mtgp_hamming_kernel(const uint32_
                 __syncwarp();
                 dirty = false;
             }
-            // the sequence holding pair p: last s with pair_base[s] <= p
-            uint32_t lo = 0, hi = n_seq;
-            while (hi - lo > 1u) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (pair_base[mid] <= p)
-                    lo = mid;
-                else
-                    hi = mid;
-            }
-            seq = lo;
-            seq_end = pair_base[lo + 1];
+            seq = lseq;
         }
-        const uint32_t* v = values + seq_start[seq] + (p - pair_base[seq]) * 2ull * K;
         uint32_t wa = 0, wb = 0;
-        // the pair's values in batches of kB per lane, all of a batch in flight
-        constexpr uint32_t kB = 16;
-        for (uint32_t j0 = 0; j0 < 2u * K; j0 += 32u * kB) {
-            uint32_t xs[kB];
+        auto weigh = [&](uint32_t j0) {
 #pragma unroll
             for (uint32_t q = 0; q < kB; ++q) {
                 const uint32_t j = j0 + 32u * q + lane;
-                xs[q] = j < 2u * K ? __ldcs(v + j) : 0u;
+                const uint32_t w = __popc(xs[q] & fmask);   // 0 past the pair's end
+                wa += j < K ? w : 0u;
+                wb += j < K ? 0u : w;
             }
+        };
+        weigh(0u);
+        if (!one)
+            for (uint32_t j0 = 32u * kB; j0 < 2u * K; j0 += 32u * kB) {
 #pragma unroll
-            for (uint32_t q = 0; q < kB; ++q) {
-                const uint32_t j = j0 + 32u * q + lane;
-                const uint32_t w = __popc(xs[q] & fmask);
-                if (j < K)
-                    wa += w;
-                else if (j < 2u * K)
-                    wb += w;
+                for (uint32_t q = 0; q < kB; ++q) {
+                    const uint32_t j = j0 + 32u * q + lane;
+                    xs[q] = j < 2u * K ? __ldcs(lv + j) : 0u;
+                }
+                weigh(j0);
             }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            wa += __shfl_xor_sync(0xFFFFFFFFu, wa, o);
-            wb += __shfl_xor_sync(0xFFFFFFFFu, wb, o);
+        if (p + 1u < p1)
+            load(p + 1u);
+        if (packed) {
+            const uint32_t s2 = __reduce_add_sync(0xFFFFFFFFu, wa | wb << 16);
+            wa = s2 & 0xFFFFu;
+            wb = s2 >> 16;
+        } else {
+            wa = __reduce_add_sync(0xFFFFFFFFu, wa);
+            wb = __reduce_add_sync(0xFFFFFFFFu, wb);
         }
         if (lane == 0) {
             uint32_t ca = 0, cb = 0;
@@ -358,11 +437,14 @@ extern "C" mtgp_status mtgp_gap_histogram(const uint32_t* values, const uint64_t
             total += counts[i];
         }
         chunk_base[n_seq] = n_chunks;
-        std::fill(hist, hist + (size_t)n_seq * (t + 1), 0ull);
-        if (total && !values)
+        if (total && !values) {
+            std::fill(hist, hist + (size_t)n_seq * (t + 1), 0ull);
             return fail(MTGP_EINVAL, "null values pointer");
-        if (n_chunks == 0)
+        }
+        if (n_chunks == 0) {   // otherwise the copy below writes every count
+            std::fill(hist, hist + (size_t)n_seq * (t + 1), 0ull);
             return ok();
+        }
         cudaStream_t s = (cudaStream_t)cuda_stream;
         Scratch sc(s);
         void *d_start, *d_counts, *d_base, *d_claim, *d_hist, *d_edges;
@@ -381,7 +463,7 @@ extern "C" mtgp_status mtgp_gap_histogram(const uint32_t* values, const uint64_t
                               cudaMemcpyHostToDevice, s), "cudaMemcpyAsync");
         Q_TRY(cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long), s), "cudaMemsetAsync");
         Q_TRY(cudaMemsetAsync(d_hist, 0, hbytes, s), "cudaMemsetAsync");
-        const size_t hsmem = (size_t)kWarps * (t + 1) * sizeof(uint32_t);   // <= 32 KB
+        const size_t hsmem = (size_t)kWarps * (t + 33) * sizeof(uint32_t);   // <= 33 KB
         const int grid = (int)std::min<uint64_t>((uint64_t)grid_for((const void*)mtgp_gap_kernel, hsmem),
                                                  (n_chunks + kWarps - 1) / kWarps);
         // chunks per claim: about four claims per warp, at most 16 chunks
@@ -431,11 +513,14 @@ extern "C" mtgp_status mtgp_hamming_pairs(const uint32_t* values, const uint64_t
             total += counts[i];
         }
         pair_base[n_seq] = pairs;
-        std::fill(table, table + (size_t)n_seq * C * C, 0ull);
-        if (total && !values)
+        if (total && !values) {
+            std::fill(table, table + (size_t)n_seq * C * C, 0ull);
             return fail(MTGP_EINVAL, "null values pointer");
-        if (pairs == 0)
+        }
+        if (pairs == 0) {   // otherwise the copy below writes every count
+            std::fill(table, table + (size_t)n_seq * C * C, 0ull);
             return ok();
+        }
         cudaStream_t st = (cudaStream_t)cuda_stream;
         Scratch sc(st);
         void *d_start, *d_base, *d_bounds, *d_table;
@@ -459,7 +544,7 @@ extern "C" mtgp_status mtgp_hamming_pairs(const uint32_t* values, const uint64_t
         mtgp_hamming_kernel<<<grid, kWarps * 32, 0, st>>>(values, (const uint64_t*)d_start,
                                                            (const uint64_t*)d_base, n_seq, pairs, fmask, K,
                                                            (const uint32_t*)d_bounds, n_bounds,
-                                                           (unsigned long long*)d_table);
+                                                           L < 65536u, (unsigned long long*)d_table);
         Q_TRY(cudaGetLastError(), "Hamming kernel launch");
         Q_TRY(cudaMemcpyAsync(table, d_table, tbytes, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync");
         Q_TRY(cudaStreamSynchronize(st), "cudaStreamSynchronize");
