@@ -3,26 +3,24 @@
 // independence (test 100) are accumulated from each sub-step's outputs
 // while they are still in registers, so the output is not read back.
 //
-// The generator is mtgp_fast_kernel's single-warp, software-pipelined row
-// loop (128-word steps, N - pos >= 256; see mtgp_fast.cuh), unchanged except
-// that the outputs of every sub-step also feed the statistics.  A sequence
+// The generator is mtgp_fast_kernel's single-warp row loop (128-word steps,
+// N - pos >= 256, tempering a row late; see gen_rows_late in mtgp_fast.cuh),
+// with the outputs of every step also feeding the statistics.  A sequence
 // of the statistics is one request of the launch (Segment::req): its values
 // in generation order.  Each request belongs to one warp, which writes its
 // histogram and table rows when the request ends.
 //
-// Gap test, per sub-step, over a run of lanes [l0, l0 + n) of one request:
-// a value visits when (value & gmask) == 0; the visits form a ballot B.  A
-// visiting lane's gap (non-visits since the previous visit) is its distance
-// to the nearest lower visiting lane, or, when there is none, lane - l0 plus
-// the carried count D of non-visits since the request's last visit (or its
-// start: the first visit's gap counts too).  Lengths >= t are pooled in
-// class t; a trailing run of non-visits is not a gap.  Each sub-step ends in
-// one shared-memory reduction per lane (red.shared.add, no return): a
-// visiting lane adds 1 to its class in the warp's histogram, the others to
-// a slot of their own that is never read, so the reduction needs neither a
-// predicate nor a branch.  In full rows the step's reductions are issued
-// after the step's row stores and warp barrier, so that they do not delay
-// them.
+// Gap test: a value visits when (value & gmask) == 0.  A gap is the number
+// of non-visits before a visit, back to the previous visit or the request's
+// start; D carries the non-visits since the last visit.  Lengths >= t are
+// pooled in class t; a trailing run of non-visits is not a gap.  Full rows
+// collect the visits of up to 32 sub-steps as ballots, one per lane, and
+// resolve them together (gap_window); other places take one sub-step, or a
+// run of lanes [l0, l0 + n) of it, at a time (gap_run).  Either way gaps are
+// counted by one shared-memory reduction per lane (red.shared.add, no
+// return): a lane with a visit adds 1 to its class in the warp's histogram,
+// the others to a slot of their own that is never read, so the reduction
+// needs neither a predicate nor a branch.
 //
 // Hamming test: the weights popc(value & hmask) of K = L/s consecutive
 // values form a block; `rem` counts the values left in the current block,
@@ -255,116 +253,217 @@ __device__ __forceinline__ uint32_t own_addr(const uint32_t* h, uint32_t lane, c
     return (uint32_t)__cvta_generic_to_shared(h + ((A.t + 1u + 3u) & ~3u) + lane);
 }
 
-// nfull consecutive full rows of one request (as gen_rows_pipelined, K = 4),
-// with the statistics of every sub-step's outputs.  STEPH: Hamming per step
+// Gap test over a window of consecutive values whose visits are spread over
+// the lanes: bit i of this lane's word w is the visit of value base + i of
+// the window, base ascending with the lane, len values in all.  Every lane
+// finds the visit before its first one (the highest lower lane with a visit,
+// or the carried run) and counts one gap per pass; lanes without a visit left
+// count in their own slot.
+__device__ __forceinline__ void gap_window(uint32_t w, uint32_t base, uint32_t len, uint32_t lane, uint32_t lower,
+                                           StatsState& st, uint32_t hs, uint32_t own, const StatsArgs& A)
+{
+    const uint32_t nz = __ballot_sync(MTGP_FULL, w != 0u);
+    if (!nz) {
+        st.D += len;
+        return;
+    }
+    const uint32_t last = base + hibit(w);   // this lane's last visit, if it has one
+    const uint32_t below = nz & lower;
+    const uint32_t pv = __shfl_sync(MTGP_FULL, last, below ? hibit(below) : 0u);
+    uint32_t next = below ? pv + 1u : 0u - st.D;   // first value after the previous visit (mod 2^32)
+    st.D = len - 1u - __shfl_sync(MTGP_FULL, last, hibit(nz));
+    while (__any_sync(MTGP_FULL, w != 0u)) {
+        const uint32_t at = base + (uint32_t)__ffs(w) - 1u;
+        count_at(w ? hs + 4u * min(at - next, A.t) : own);
+        w &= w - 1u;
+        next = at + 1u;
+    }
+}
+
+// Hamming test over one step's outputs (KS sub-steps, step_n values in lane
+// order; w = this lane's weights), K >= 128: at most one block end.
+template <int KS>
+__device__ __forceinline__ void ham_step(const uint32_t (&w)[4], uint32_t step_n, uint32_t lane, StatsState& st,
+                                         uint32_t* tab, const StatsArgs& A)
+{
+    if (st.rem > step_n) {
+        uint32_t a = st.acc;
+#pragma unroll
+        for (int i = 0; i < KS; ++i)
+            a += w[i];
+        st.acc = a;
+        st.rem -= step_n;
+    } else {
+        // the block ends inside this step: step positions >= rem belong to
+        // the next block
+        uint32_t cur = st.acc, nxt = 0u;
+#pragma unroll
+        for (int i = 0; i < KS; ++i) {
+            const bool after = 32u * (uint32_t)i + lane >= st.rem;
+            cur += after ? 0u : w[i];
+            nxt += after ? w[i] : 0u;
+        }
+        const uint32_t W = __reduce_add_sync(MTGP_FULL, cur);
+        st.acc = nxt;
+        block_done(W, lane, st, tab, A);
+        st.rem = st.rem + A.K - step_n;
+    }
+}
+
+// nfull consecutive full rows of one request: the loop of gen_rows_late with
+// the statistics of every step's outputs, a row late like the outputs.  Row q
+// of the run gives the numbers (q-1)N+1 .. qN (row 0: number 0 alone), the
+// last row's other numbers follow after the loop.  STEPH: Hamming per step
 // (K >= 128), else per sub-step.
+//
+// The gap test keeps each sub-step's visits as a ballot in one lane and
+// resolves a window of up to 32 of them at once (two rows for up to 16 column
+// groups, one row for up to 32, half a row beyond): three instructions per 32
+// numbers and about 60 per window.  Resolved per sub-step, the test took 15
+// instructions and a shared reduction per 32 numbers and was the largest part
+// of the loop.  Measured (one launch, 5.12 G numbers, Mexp 11213): 14.0 -> 10.6
+// ms at 8 warps per SM, 10.3 -> 7.35 ms at 16 split in pieces of 1 052 897;
+// 2432 x 2^19 at Mexp 23209 and 16 warps per SM 2.44 -> 1.94 ms, at Mexp 44497
+// and 8 3.61 -> 2.53 ms (its registers leave no room for 16).  What bounds it:
+// issue and latency, about 165 instructions per 128 numbers.
 template <int M, int FMT, bool STEPH>
-__device__ __forceinline__ void fused_rows(uint32_t (&r)[M], uint32_t* Sw, uint32_t* ow, const uint32_t* Q,
-                                           const RowP& P, uint32_t lane, const uint32_t* __restrict__ Tb,
-                                           uint32_t last_lane, uint32_t nfull, StatsState& st, uint32_t* h,
-                                           uint32_t* tab, const StatsArgs& A)
+__device__ __forceinline__ void fused_rows(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
+                                           const uint32_t* __restrict__ Tb, uint32_t nfull, StatsState& st,
+                                           uint32_t* h, uint32_t* tab, const StatsArgs& A)
 {
     constexpr int K = 4;
     constexpr int NS = (M + K - 1) / K;
-    const uint32_t N = P.n;
+    constexpr int TT = FMT == 0 ? 64 : 128;
+    constexpr int RB = M <= 16 ? 2 : 1;   // rows per gap window (M <= 32)
+    const uint32_t N = P.n, last_lane = (N - 1u) & 31u, nlast = last_lane + 1u;
     const uint32_t lower = (1u << lane) - 1u;
-    const bool last_ok = lane <= last_lane;     // lane holds a column of the row's last group
-    const uint32_t nlast = last_lane + 1u;      // columns of the last group
-    const uint32_t hs = hist_addr(h);
-    const uint32_t own = own_addr(h, lane, A);
-    uint32_t x1[K], xp[K], xq[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-        x1[i] = Sw[32 * i + 1];
-        xp[i] = Q[32 * i];
-        xq[i] = Q[32 * i - 1];
-    }
-    for (uint32_t q = 0; q < nfull; ++q, ow += N) {
-#pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            const int s0 = s * K;
-            const int n0 = (s + 1 < NS) ? s0 + K : 0;
-            uint32_t y1[K], yp[K], yq[K];
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                if (n0 + i < M) {
-                    y1[i] = Sw[32 * (n0 + i) + 1];
-                    yp[i] = Q[32 * (n0 + i)];
-                    yq[i] = Q[32 * (n0 + i) - 1];
+    const uint32_t hs = hist_addr(h), own = own_addr(h, lane, A);
+    uint32_t sa = saddr(S + lane);
+    uint32_t x1_last = lane >= last_lane ? saddr(S) : sa + 128u * (M - 1) + 4u;
+    uint32_t tb = saddr(Tb);
+    uint32_t mul1 = 1u << P.sh1;   // on the FMA pipe, as in gen_rows_late
+    asm volatile("" : "+r"(mul1), "+r"(sa), "+r"(x1_last), "+r"(tb));
+    uint32_t r[M], qa[M], T[NS];
+    static_for<M>([&](auto im) {
+        constexpr int m = im.value;
+        const uint32_t p = 32u * m + lane + P.pos;
+        r[m] = lds_at<128 * m>(sa);
+        qa[m] = saddr(S + (p < N ? p : p - N));
+        asm volatile("" : "+r"(qa[m]));
+    });
+    static_for<NS>([&](auto is) { T[is.value] = 0u; });
+    T[NS - 1] = (temper_index(S[P.pos - 1u]) & 15u) << (2 + 8 * ((M - 1) & 3));
+    uint32_t x1[K], xp[K];
+    static_for<K>([&](auto ii) {
+        constexpr int i = ii.value;
+        x1[i] = lds_at<128 * i + 4>(sa);
+        xp[i] = lds_at<0>(qa[i]);
+    });
+    uint32_t* op = ow + 1 - (int)N;
+    // the gap window: this lane's ballot, its place in the window, rows in it
+    uint32_t vw = 0u, rb = 0u, slot = lane;   // slot: lane less the window's earlier groups
+    const uint32_t base = M <= 32 ? (lane / (uint32_t)M) * N + 32u * (lane % (uint32_t)M) : 32u * lane;
+#pragma unroll 1
+    for (uint32_t q = 0; q < nfull; ++q, op += N) {
+        const bool body = q != 0u;
+        static_for<NS>([&](auto is) {
+            constexpr int s = is.value, s0 = s * K;
+            constexpr int n0 = (s + 1 < NS) ? s0 + K : 0;
+            constexpr int KS = (M - s0 < K) ? M - s0 : K;   // sub-steps of this step
+            constexpr bool lasts = s0 + KS == M;
+            uint32_t y1[K], yp[K], xn[K], o[K], tw[K], w[K];
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value, m = n0 + i;
+                if constexpr (m < M) {
+                    if constexpr (m + 1 < M)
+                        y1[i] = lds_at<128 * m + 4>(sa);
+                    else
+                        y1[i] = lds_at<0>(x1_last);
+                    yp[i] = lds_at<0>(qa[m]);
                 }
-            }
-            uint32_t xn[K], o[K], w[K], ad[K];
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                if (s0 + i < M) {
-                    const uint32_t yy = (r[s0 + i] & P.mask) ^ x1[i];
-                    const uint32_t y = yy ^ (yy << P.sh1) ^ (xp[i] >> P.sh2);
-                    xn[i] = y ^ tbl(Tb, 0u, y);
-                    o[i] = temper_convert<FMT>(xn[i], temper_index(xq[i]), Tb);
-                }
-            }
-            // statistics of this step's outputs
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                if (s0 + i < M) {
-                    const bool lastg = s0 + i + 1 == M;
-                    const bool valid = !lastg || last_ok;
-                    ad[i] = gap_run(o[i], valid, 0u, lastg ? nlast : 32u, lane, lower, st, hs, own, A);
+            });
+            static_for<KS>([&](auto ii) {
+                constexpr int i = ii.value;
+                tw[i] = lds_at<TT>(__byte_perm(T[s], tb, 0x7650 + i));
+            });
+            T[s] = temper_pack(xp);
+            static_for<KS>([&](auto ii) {
+                constexpr int i = ii.value, m = s0 + i;
+                const uint32_t yy = (r[m] & P.mask) ^ x1[i];
+                const uint32_t y = yy ^ (yy * mul1) ^ (xp[i] >> P.sh2);
+                xn[i] = y ^ tbl(Tb, 0u, y);
+                o[i] = finish<FMT>(x1[i], tw[i]);
+            });
+            static_for<KS>([&](auto ii) {
+                constexpr int i = ii.value, m = s0 + i;
+                r[m] = xn[i];
+                sts_at<128 * m>(sa, xn[i]);
+            });
+            __syncwarp();
+            if (body) {
+                static_for<KS>([&](auto ii) {
+                    constexpr int i = ii.value, m = s0 + i;
+                    const bool valid = m + 1 < M || lane <= last_lane;
+                    if (valid)
+                        __stcs(op + 32 * m, o[i]);
+                    const uint32_t B = __ballot_sync(MTGP_FULL, valid && (o[i] & A.gmask) == 0u);
+                    vw = slot == (uint32_t)(M <= 32 ? m : m & 31) ? B : vw;
                     w[i] = valid ? __popc(o[i] & A.hmask) : 0u;
                     if constexpr (!STEPH)
-                        ham_run(w[i], 0u, lastg ? nlast : 32u, lane, st, tab, A);
+                        ham_run(w[i], 0u, m + 1 < M ? 32u : nlast, lane, st, tab, A);
+                });
+                if constexpr (STEPH)
+                    ham_step<KS>(w, lasts ? 32u * (KS - 1) + nlast : 32u * KS, lane, st, tab, A);
+                if constexpr (M > 32 && s0 + KS == 32) {
+                    gap_window(vw, base, 1024u, lane, lower, st, hs, own, A);
+                    vw = 0u;
                 }
-            }
-            if constexpr (STEPH) {
-                const int KS = (M - s0 < K) ? M - s0 : K;   // sub-steps in this step
-                const uint32_t step_n = (s0 + KS == M) ? 32u * (KS - 1) + nlast : 32u * KS;
-                if (st.rem > step_n) {
-                    uint32_t a = st.acc;
-#pragma unroll
-                    for (int i = 0; i < KS; ++i)
-                        a += w[i];
-                    st.acc = a;
-                    st.rem -= step_n;
-                } else {
-                    // the block ends inside this step: step positions >= rem
-                    // belong to the next block
-                    uint32_t cur = st.acc, nxt = 0u;
-#pragma unroll
-                    for (int i = 0; i < KS; ++i) {
-                        const bool after = 32u * (uint32_t)i + lane >= st.rem;
-                        cur += after ? 0u : w[i];
-                        nxt += after ? w[i] : 0u;
+                if constexpr (lasts && M > 32) {
+                    gap_window(vw, base, N - 1024u, lane, lower, st, hs, own, A);
+                    vw = 0u;
+                }
+                if constexpr (lasts && M <= 32) {
+                    slot -= (uint32_t)M;
+                    if (++rb == (uint32_t)RB) {
+                        gap_window(vw, base, RB * N, lane, lower, st, hs, own, A);
+                        vw = rb = 0u;
+                        slot = lane;
                     }
-                    const uint32_t W = __reduce_add_sync(MTGP_FULL, cur);
-                    st.acc = nxt;
-                    block_done(W, lane, st, tab, A);
-                    st.rem = st.rem + A.K - step_n;
                 }
+            } else if constexpr (lasts) {
+                // number 0 of the run, at column N-1
+                constexpr int i = M - 1 - s0;
+                const bool valid = lane == last_lane;
+                if (valid)
+                    __stcs(op + 32 * (M - 1), o[i]);
+                count_at(gap_run(o[i], valid, last_lane, 1u, lane, lower, st, hs, own, A));
+                ham_run(valid ? __popc(o[i] & A.hmask) : 0u, last_lane, 1u, lane, st, tab, A);
             }
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const int m = s0 + i;
-                if (m < M && (m + 1 < M || last_ok)) {
-                    r[m] = xn[i];
-                    Sw[32 * m] = xn[i];
-                    if (32u * (uint32_t)m < P.mirror)
-                        Sw[32 * m + N] = xn[i];
-                    __stcs(ow + 32 * m, o[i]);
-                }
-            }
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                if (s0 + i < M)
-                    count_at(ad[i]);
-                if (n0 + i < M) {
+            static_for<K>([&](auto ii) {
+                constexpr int i = ii.value;
+                if constexpr (n0 + i < M) {
                     x1[i] = y1[i];
                     xp[i] = yp[i];
-                    xq[i] = yq[i];
                 }
-            }
-        }
+            });
+        });
     }
+    if (rb)
+        gap_window(vw, base, rb * N, lane, lower, st, hs, own, A);
+    // the last row's numbers after its first, one sub-step at a time
+    static_for<M>([&](auto im) {
+        constexpr int m = im.value;
+        const uint32_t n = m + 1 < M ? 32u : last_lane;
+        const bool valid = lane < n;
+        const uint32_t tw = lds_at<TT>(__byte_perm(T[m / K], tb, 0x7650 + m % K));
+        const uint32_t o = finish<FMT>(lds_at<128 * m + 4>(sa), tw);
+        if (n) {
+            if (valid)
+                __stcs(op + 32 * m, o);
+            count_at(gap_run(o, valid, 0u, n, lane, lower, st, hs, own, A));
+            ham_run(valid ? __popc(o & A.hmask) : 0u, 0u, n, lane, st, tab, A);
+        }
+    });
 }
 
 // nfull consecutive full rows of one request for short states (M < 9, no
@@ -374,28 +473,38 @@ __device__ __forceinline__ void fused_rows(uint32_t (&r)[M], uint32_t* Sw, uint3
 // N - pos >= 64: none of them is written by this sub-step, and a wrapped
 // pick-up lands on a column of an earlier, already written sub-step.
 template <int M, int FMT>
-__device__ __forceinline__ void fused_rows_short(uint32_t (&r)[M], uint32_t* Sw, uint32_t* ow, const uint32_t* Q,
-                                                 const RowP& P, uint32_t lane, const uint32_t* __restrict__ Tb,
-                                                 uint32_t last_lane, uint32_t nfull, StatsState& st, uint32_t* h,
-                                                 uint32_t* tab, const StatsArgs& A)
+__device__ __forceinline__ void fused_rows_short(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
+                                                 const uint32_t* __restrict__ Tb, uint32_t nfull, StatsState& st,
+                                                 uint32_t* h, uint32_t* tab, const StatsArgs& A)
 {
     static_assert(M >= 3, "the look-ahead read of the last sub-step needs three column groups");
-    const uint32_t N = P.n;
+    const uint32_t N = P.n, last_lane = (N - 1u) & 31u;
     const uint32_t lower = (1u << lane) - 1u;
     const bool last_ok = lane <= last_lane;
     const uint32_t nlast = last_lane + 1u;
     const uint32_t hs = hist_addr(h);
     const uint32_t own = own_addr(h, lane, A);
+    uint32_t* const Sw = S + lane;
+    uint32_t r[M];
+    const uint32_t *Qp[M], *Qq[M];   // words i+pos and i+pos-1, with the wrap at column N in the address
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const uint32_t p = 32u * (uint32_t)m + lane + P.pos;
+        r[m] = Sw[32 * m];
+        Qp[m] = S + (p < N ? p : p - N);
+        Qq[m] = S + (p - 1u < N ? p - 1u : p - 1u - N);
+    }
+    const uint32_t* const x1_last = lane >= last_lane ? S : Sw + (32 * (M - 1) + 1);
     uint32_t x1 = Sw[1];
-    uint32_t xp = Q[0];
-    uint32_t xq = Q[-1];
+    uint32_t xp = *Qp[0];
+    uint32_t xq = *Qq[0];
     for (uint32_t q = 0; q < nfull; ++q, ow += N) {
 #pragma unroll
         for (int m = 0; m < M; ++m) {
             const int mn = m + 1 < M ? m + 1 : 0;   // the next sub-step (of the next row after the last)
-            const uint32_t y1 = Sw[32 * mn + 1];
-            const uint32_t yp = Q[32 * mn];
-            const uint32_t yq = Q[32 * mn - 1];
+            const uint32_t y1 = mn + 1 < M ? Sw[32 * mn + 1] : *x1_last;
+            const uint32_t yp = *Qp[mn];
+            const uint32_t yq = *Qq[mn];
             const uint32_t yy = (r[m] & P.mask) ^ x1;
             const uint32_t y = yy ^ (yy << P.sh1) ^ (xp >> P.sh2);
             const uint32_t xn = y ^ tbl(Tb, 0u, y);
@@ -408,8 +517,6 @@ __device__ __forceinline__ void fused_rows_short(uint32_t (&r)[M], uint32_t* Sw,
             if (valid) {
                 r[m] = xn;
                 Sw[32 * m] = xn;
-                if (32u * (uint32_t)m < P.mirror)
-                    Sw[32 * m + N] = xn;
                 __stcs(ow + 32 * m, o);
             }
             __syncwarp();
@@ -425,29 +532,25 @@ __device__ __forceinline__ void fused_rows_short(uint32_t (&r)[M], uint32_t* Sw,
 // columns): each lane finds its request; the statistics take the row's
 // sub-steps in order, one run of same-request lanes at a time.
 template <int M>
-__device__ __forceinline__ void fused_row_slow(uint32_t (&r)[M], uint32_t* Sw, const uint32_t* Q,
-                                               const RowP& P, uint32_t lane,
+__device__ __forceinline__ void fused_row_slow(uint32_t* S, const RowP& P, uint32_t lane,
                                                const uint32_t* __restrict__ Tb, uint32_t n_valid,
                                                uint64_t row_g, const Segment* __restrict__ segs,
                                                uint32_t s_first, uint32_t s_end, uint32_t* __restrict__ out,
                                                StatsState& st, uint32_t* h, uint32_t* tab, const StatsArgs& A)
 {
-    const uint32_t lower = (1u << lane) - 1u;
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        if (32u * (uint32_t)m >= n_valid)
-            break;
-        const int off = 32 * m;
-        const uint32_t x1 = Sw[off + 1];
-        const uint32_t xp = Q[off];
-        const uint32_t xq = Q[off - 1];
-        const uint32_t yy = (r[m] & P.mask) ^ x1;
+    const uint32_t lower = (1u << lane) - 1u, N = P.n;
+#pragma unroll 1
+    for (uint32_t c0 = 0; c0 < n_valid; c0 += 32u) {
+        const uint32_t col = c0 + lane, p = col + P.pos, pw = p < N ? p : p - N;
+        const uint32_t x1 = S[col + 1u == N ? 0u : col + 1u];
+        const uint32_t xp = S[pw];
+        const uint32_t xq = S[pw ? pw - 1u : N - 1u];
+        const uint32_t yy = (S[col] & P.mask) ^ x1;
         const uint32_t y = yy ^ (yy << P.sh1) ^ (xp >> P.sh2);
         const uint32_t xn = y ^ tbl(Tb, 0u, y);
         const uint32_t ti = temper_index(xq);
         const uint32_t ou = temper_convert<0>(xn, ti, Tb);
         const uint32_t of = temper_convert<1>(xn, ti, Tb);
-        const uint32_t col = 32u * (uint32_t)m + lane;
         const bool valid = col < n_valid;
         // this lane's request and stored value
         uint32_t s = s_first;
@@ -476,10 +579,7 @@ __device__ __forceinline__ void fused_row_slow(uint32_t (&r)[M], uint32_t* Sw, c
         }
         __syncwarp();
         if (valid) {
-            r[m] = xn;
-            Sw[off] = xn;
-            if (32u * (uint32_t)m < P.mirror)
-                Sw[off + P.n] = xn;
+            S[col] = xn;
             out[sg.out_off + (gi - sg.g_start)] = o;
         }
         __syncwarp();
@@ -496,24 +596,10 @@ __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uin
                                            uint32_t* tab, const StatsArgs& A)
 {
     const uint32_t N = P.n;
-    const uint32_t last_lane = (N - 1u) & 31u;
     for (uint32_t c = lane; c < (KP.np >> 2); c += 32u)
         cp_async16(S + 4u * c, g + 4u * c);
     cp_async_wait_all();
     __syncwarp();
-    uint32_t r[M];
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-        const uint32_t c = 32u * (uint32_t)j + lane;
-        r[j] = c < N ? S[c] : 0u;
-    }
-    for (uint32_t c = lane; c < P.mirror; c += 32u) {
-        const uint32_t v = S[c];
-        S[N + c] = v;
-    }
-    __syncwarp();
-    uint32_t* Sw = S + lane;
-    const uint32_t* Q = S + P.pos + lane;
     const Segment last = segs[s_end - 1u];
     const uint64_t total = last.g_start + last.count;
     uint32_t s = s_begin;
@@ -533,37 +619,37 @@ __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uin
                 // a piece whose first gap or first pair is still open: one row
                 // at a time on the slow path, which records them (also short
                 // states too close for the look-ahead read, N - pos < 64)
-                fused_row_slow<M>(r, Sw, Q, P, lane, Tb, N, row, segs, s, s_end, out, st, h, tab, A);
+                fused_row_slow<M>(S, P, lane, Tb, N, row, segs, s, s_end, out, st, h, tab, A);
                 row += N;
                 continue;
             }
             if constexpr (M < 9) {
                 if (sg.fmt == 0)
-                    fused_rows_short<M, 0>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows_short<M, 0>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else if (sg.fmt == 1)
-                    fused_rows_short<M, 1>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows_short<M, 1>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else
-                    fused_rows_short<M, 2>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows_short<M, 2>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
             } else if (A.K >= 128u) {
                 if (sg.fmt == 0)
-                    fused_rows<M, 0, true>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows<M, 0, true>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else if (sg.fmt == 1)
-                    fused_rows<M, 1, true>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows<M, 1, true>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else
-                    fused_rows<M, 2, true>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows<M, 2, true>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
             } else {
                 if (sg.fmt == 0)
-                    fused_rows<M, 0, false>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows<M, 0, false>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else if (sg.fmt == 1)
-                    fused_rows<M, 1, false>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows<M, 1, false>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else
-                    fused_rows<M, 2, false>(r, Sw, ow, Q, P, lane, Tb, last_lane, nfull, st, h, tab, A);
+                    fused_rows<M, 2, false>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
             }
             row += (uint64_t)nfull * N;
         } else {
             const uint64_t left = total - row;
             const uint32_t n_valid = left < (uint64_t)N ? (uint32_t)left : N;
-            fused_row_slow<M>(r, Sw, Q, P, lane, Tb, n_valid, row, segs, s, s_end, out, st, h, tab, A);
+            fused_row_slow<M>(S, P, lane, Tb, n_valid, row, segs, s, s_end, out, st, h, tab, A);
             row += N;
         }
     }
@@ -579,7 +665,7 @@ __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uin
 // Persistent kernel: every warp claims streams (longest first) from the
 // work table and advances each alone, with the statistics.
 template <int M, int G>
-__global__ void __launch_bounds__(G * 32) mtgp_fused_kernel(const KParams P, uint32_t* __restrict__ states,
+__global__ void __launch_bounds__(G * 32, M < 32 ? 2 : 1) mtgp_fused_kernel(const KParams P, uint32_t* __restrict__ states,
                                                             uint32_t n_streams,
                                                             const WorkItem* __restrict__ items,
                                                             const Segment* __restrict__ segs,
@@ -590,7 +676,7 @@ __global__ void __launch_bounds__(G * 32) mtgp_fused_kernel(const KParams P, uin
                                                             const StatsArgs A)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ __align__(64) uint32_t Tb[G][48];
+    __shared__ __align__(256) uint32_t Tb[G][64];   // as in mtgp_fast_kernel
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = threadIdx.x >> 5;
     if (threadIdx.x < 16) {

@@ -6,6 +6,7 @@
 namespace mtgp {
 
 const void* fused_ptr_group_b(int M, int G);
+const void* fused_ptr_group_c(int M, int G);
 
 static const void* fused_ptr_group_a(int M, int G)
 {
@@ -20,7 +21,9 @@ static const void* fused_ptr_group_a(int M, int G)
 const void* fused_kernel_ptr(int M, int G)
 {
     const void* p = fused_ptr_group_a(M, G);
-    return p ? p : fused_ptr_group_b(M, G);
+    if (!p)
+        p = fused_ptr_group_b(M, G);
+    return p ? p : fused_ptr_group_c(M, G);
 }
 
 cudaError_t launch_fused(const void* fn, const GenArgs& a, const StatsArgs& A, dim3 grid, dim3 block,
