@@ -426,9 +426,10 @@ mtgp_status mtgp::split_work(const Work& w, uint64_t max_piece, uint32_t max_pie
         std::vector<Segment> segs;
     };
     std::vector<Piece> pieces;
-    auto new_row = [&](uint32_t stream) -> uint32_t {
+    auto new_row = [&](uint32_t stream, bool jumped) -> uint32_t {
         const uint32_t row = o.n_rows++;
-        o.copies.push_back(make_uint2(stream, row));
+        if (!jumped)
+            o.copies.push_back(make_uint2(stream, row));
         o.row_set.push_back(set_of_stream.empty() ? 0u : set_of_stream[stream]);
         return row;
     };
@@ -440,7 +441,7 @@ mtgp_status mtgp::split_work(const Work& w, uint64_t max_piece, uint32_t max_pie
             return fail(MTGP_EINVAL, "too many pieces");
         if (T <= max_piece) {
             Piece p{it, T, std::vector<Segment>(sg, sg + it.nseg)};
-            p.it.stream = new_row(it.stream);
+            p.it.stream = new_row(it.stream, false);
             o.backs.push_back(make_uint2(p.it.stream, it.stream));
             pieces.push_back(std::move(p));
             continue;
@@ -457,10 +458,11 @@ mtgp_status mtgp::split_work(const Work& w, uint64_t max_piece, uint32_t max_pie
             const uint64_t lo = j * L, hi = std::min(T, lo + L);
             Piece p;
             p.it = it;
-            p.it.stream = new_row(it.stream);
+            p.it.stream = new_row(it.stream, j > 0);
             p.total = hi - lo;
             if (j > 0) {
                 o.jump_rows.push_back(p.it.stream);
+                o.jump_src.push_back(it.stream);
                 o.jump_sets.push_back(o.row_set.back());
                 o.jump_lens.push_back(lo);
             }
@@ -1382,12 +1384,12 @@ static mtgp_status record_graph(mtgp_plan* p)
     const uint32_t n_jumps = (uint32_t)p->jumps.items.size();
     const bool split = p->split.n_rows > 0;
     CUDA_TRY(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
-    // split launches: every row gets its stream's state, then the rows of
-    // later pieces are jumped to their offsets
+    // split launches: every row gets its stream's state, the rows of later
+    // pieces advanced to their offsets
     cudaError_t e1 = launch_copy_rows(p->st->d_states, p->d_rows, p->d_copies, n_copies,
                                       p->st->P.k.n, p->st->P.k.np, cap);
     if (e1 == cudaSuccess)
-        e1 = launch_jump_batch(p->st, p->d_rows, p->d_jitems, n_jumps, p->d_jpolys, p->jumps.words,
+        e1 = launch_jump_batch(p->st, p->st->d_states, p->d_rows, p->d_jitems, n_jumps, p->d_jpolys, p->jumps.words,
                                p->jumps.smem, cap);
     GenArgs a;
     a.P = p->st->P.k;
@@ -1488,9 +1490,10 @@ static mtgp_status build_launch(mtgp_plan* p, uint64_t max_piece)
     if (r != MTGP_OK)
         return r;
     JumpBatch jb;
-    r = build_jump_batch(st, sw.jump_rows, sw.jump_sets, sw.jump_lens, &jb);
+    r = build_jump_batch(st, sw.jump_rows, sw.jump_src, sw.jump_sets, sw.jump_lens, &jb);
     if (r != MTGP_OK)
         return r;
+    fold_copies(&sw, &jb);
     CUDA_TRY(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
     free_split(p);
     if (p->d_table) {
@@ -1510,9 +1513,11 @@ static mtgp_status build_launch(mtgp_plan* p, uint64_t max_piece)
             CUDA_TRY(cudaMemcpy(p->d_row_set, sw.row_set.data(), sw.row_set.size() * 4,
                                 cudaMemcpyHostToDevice), "cudaMemcpy(row sets)");
         }
-        CUDA_TRY(cudaMalloc(&p->d_copies, sw.copies.size() * sizeof(uint2)), "cudaMalloc(copy pairs)");
-        CUDA_TRY(cudaMemcpy(p->d_copies, sw.copies.data(), sw.copies.size() * sizeof(uint2),
-                            cudaMemcpyHostToDevice), "cudaMemcpy(copy pairs)");
+        if (!sw.copies.empty()) {
+            CUDA_TRY(cudaMalloc(&p->d_copies, sw.copies.size() * sizeof(uint2)), "cudaMalloc(copy pairs)");
+            CUDA_TRY(cudaMemcpy(p->d_copies, sw.copies.data(), sw.copies.size() * sizeof(uint2),
+                                cudaMemcpyHostToDevice), "cudaMemcpy(copy pairs)");
+        }
         CUDA_TRY(cudaMalloc(&p->d_backs, sw.backs.size() * sizeof(uint2)), "cudaMalloc(copy-back pairs)");
         CUDA_TRY(cudaMemcpy(p->d_backs, sw.backs.data(), sw.backs.size() * sizeof(uint2),
                             cudaMemcpyHostToDevice), "cudaMemcpy(copy-back pairs)");
@@ -1971,7 +1976,7 @@ extern "C" mtgp_status mtgp_plan_get_info(mtgp_plan_t p, mtgp_plan_info* info)
     info->max_piece = p->split.max_piece;
     info->n_split_streams = p->split.n_split;
     info->n_pieces = p->split.n_pieces;
-    info->n_jumps = (uint32_t)p->jumps.items.size();
+    info->n_jumps = (uint32_t)p->jumps.items.size() - p->jumps.n_copies;
     info->kernel_launches = p->kernel_launches;
     const Geometry& geo = p->stats ? p->stats_geo : p->geo;
     LaunchCfg eff = p->cfg;

@@ -127,15 +127,18 @@ struct GenArgs {
     const uint32_t* set_of = nullptr;  // set index of each stream when `sets` is given
 };
 
-// Jump of one state row by a count J: row `stream` of the array given to the
-// launch, polynomial `poly` of the launch's table (degree `deg`), parameter
-// set `set` (per-stream sets) or 0.
+// Jump of one state row by a count J: from row `src` of the array a launch
+// reads to row `stream` of the one it writes, polynomial `poly` of the
+// launch's table (degree `deg`, or kCopyRow: the row is copied), parameter set
+// `set` (per-stream sets) or 0.
 struct JumpItem {
     uint32_t stream;
+    uint32_t src;
     uint32_t poly;
     uint32_t deg;
     uint32_t set;
 };
+constexpr uint32_t kCopyRow = 0xFFFFFFFFu;
 
 // Copies state rows: dst[pairs[i].y] = src[pairs[i].x], N words each (row
 // stride np).

@@ -468,7 +468,7 @@ __device__ __forceinline__ void jump_block16(uint32_t bits, const uint32_t* y, u
 // bits whose window would reach past it go bit by bit.
 template <int UC>
 __global__ void __launch_bounds__(32 * kJumpWarps) mtgp_jump_kernel(
-    const KParams P, uint32_t* __restrict__ states, const JumpItem* __restrict__ items,
+    const KParams P, const uint32_t* from, uint32_t* states, const JumpItem* __restrict__ items,
     const uint32_t* __restrict__ polys, uint32_t poly_words, const KSet* __restrict__ sets, uint32_t s_len)
 {
     extern __shared__ __align__(16) uint32_t sm[];
@@ -476,6 +476,14 @@ __global__ void __launch_bounds__(32 * kJumpWarps) mtgp_jump_kernel(
     const uint32_t part = cluster.block_rank(), parts = cluster.num_blocks();
     const JumpItem it = items[blockIdx.x / parts];
     const uint32_t N = P.n, D = it.deg + 1u;
+    const uint32_t* f = from + (size_t)it.src * P.np;
+    uint32_t* g = states + (size_t)it.stream * P.np;
+    if (it.deg == kCopyRow) {   // every CTA of the cluster leaves here
+        if (part == 0u)
+            for (uint32_t j = threadIdx.x; j < N; j += blockDim.x)
+                g[j] = f[j];
+        return;
+    }
     uint32_t pos = P.pos, sh1 = P.sh1, sh2 = P.sh2;
     const uint32_t* rec = P.rec;
     if (sets) {
@@ -490,9 +498,8 @@ __global__ void __launch_bounds__(32 * kJumpWarps) mtgp_jump_kernel(
     __shared__ uint32_t R[16];
     if (threadIdx.x < 16)
         R[threadIdx.x] = rec[threadIdx.x];
-    uint32_t* g = states + (size_t)it.stream * P.np;
     for (uint32_t j = threadIdx.x; j < N; j += blockDim.x) {
-        S[j] = g[j];
+        S[j] = f[j];
         acc[j] = 0u;
     }
     __syncthreads();
@@ -913,10 +920,11 @@ static std::vector<const Poly*> jump_polys(const SetP& p, const Poly& mu, const 
 }
 
 mtgp_status mtgp::build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>& rows,
-                                   const std::vector<uint32_t>& sets, const std::vector<uint64_t>& jumps,
+                                   const std::vector<uint32_t>& srcs, const std::vector<uint32_t>& sets, const std::vector<uint64_t>& jumps,
                                    JumpBatch* out, const std::vector<KSet>* given_sets)
 {
     out->items.clear();
+    out->n_copies = 0;
     out->poly_words.clear();
     out->words = 0;
     out->smem = 0;
@@ -964,6 +972,7 @@ mtgp_status mtgp::build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>
         }
         prev = i;
         ji.stream = rows[i];
+        ji.src = srcs[i];
         out->items.push_back(ji);
     }
     if (out->items.empty())
@@ -1000,16 +1009,34 @@ mtgp_status mtgp::build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>
     return MTGP_OK;
 }
 
-cudaError_t mtgp::launch_jump_batch(const mtgp_streams* st, uint32_t* rows_base, const JumpItem* d_items,
+void mtgp::fold_copies(SplitWork* sw, JumpBatch* jb)
+{
+    // A CTA of the jump kernel takes a copy in about the time a launch of the
+    // copy kernel takes to start, so only launches with few copies fold them.
+    if (jb->items.empty() || sw->copies.size() > 64)
+        return;
+    for (const uint2& c : sw->copies)
+        jb->items.push_back(JumpItem{c.y, c.x, 0u, kCopyRow, 0u});
+    jb->n_copies = (uint32_t)sw->copies.size();
+    sw->copies.clear();
+}
+
+cudaError_t mtgp::launch_jump_batch(const mtgp_streams* st, const uint32_t* from, uint32_t* rows_base,
+                                    const JumpItem* d_items,
                                     uint32_t n, const uint32_t* d_polys, uint32_t words, size_t smem,
                                     cudaStream_t s)
 {
     if (n == 0)
         return cudaSuccess;
     // Few jumps leave most of the chip idle, so each is shared out over a
-    // cluster of up to 8 CTAs, as long as every CTA still has an SM to itself.
+    // cluster of up to 8 CTAs, as long as there are no more than two CTAs
+    // (32 warps) per SM.  Measured at Mexp 11213 and 23209, whole calls: 63
+    // jumps 53 -> 51 and 92 -> 86 us against one CTA per SM, 152 jumps 66 ->
+    // 62 and 142 -> 118; four per SM is slower again (81 and 152).
+    // 10 000 jumps at Mexp 11213 take 1.21 ms, 18 SM-us each (56 before the
+    // sliding windows): 117 000 warp instructions, issue 76 % busy.
     uint32_t parts = 1;
-    while (parts < 8u && 2u * parts * n <= (uint32_t)st->sms)
+    while (parts < 8u && parts * n <= (uint32_t)st->sms)
         parts *= 2u;
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(n * parts);
@@ -1026,7 +1053,7 @@ cudaError_t mtgp::launch_jump_batch(const mtgp_streams* st, uint32_t* rows_base,
     KParams P = st->P.k;
     const KSet* sets = st->d_sets;
     uint32_t s_len = (uint32_t)(smem / 4u) - P.n;
-    void* args[] = {&P, &rows_base, (void*)&d_items, (void*)&d_polys, &words, (void*)&sets, &s_len};
+    void* args[] = {&P, (void*)&from, &rows_base, (void*)&d_items, (void*)&d_polys, &words, (void*)&sets, &s_len};
     return cudaLaunchKernelExC(&c, jump_fn(P.n), args);
 }
 
@@ -1082,7 +1109,7 @@ extern "C" mtgp_status mtgp_jump(mtgp_streams_t st, const uint32_t* ids, const u
             lens.push_back(kv.second);
         }
         JumpBatch b;
-        mtgp_status r = build_jump_batch(st, rows, sets, lens, &b);
+        mtgp_status r = build_jump_batch(st, rows, rows, sets, lens, &b);
         if (r != MTGP_OK)
             return r;
         if (b.items.empty())
@@ -1100,7 +1127,7 @@ extern "C" mtgp_status mtgp_jump(mtgp_streams_t st, const uint32_t* ids, const u
         std::memcpy(sl.host, b.items.data(), b_items);
         std::memcpy((char*)sl.host + o_poly, b.poly_words.data(), b.poly_words.size() * 4u);
         J_TRY(cudaMemcpyAsync(sl.dev, sl.host, bytes, cudaMemcpyHostToDevice, cs), "cudaMemcpyAsync(jumps)");
-        J_TRY(launch_jump_batch(st, st->d_states, (const JumpItem*)sl.dev, (uint32_t)b.items.size(),
+        J_TRY(launch_jump_batch(st, st->d_states, st->d_states, (const JumpItem*)sl.dev, (uint32_t)b.items.size(),
                                 (const uint32_t*)((char*)sl.dev + o_poly), b.words, b.smem, cs), "jump kernel");
         J_TRY(cudaEventRecord(sl.ev, cs), "cudaEventRecord");
         sl.ev_recorded = true;

@@ -115,6 +115,7 @@ namespace mtgp {
 // shared memory.
 struct JumpBatch {
     std::vector<JumpItem> items;
+    uint32_t n_copies = 0;   // of the items: plain copies (fold_copies)
     std::vector<uint32_t> poly_words;
     uint32_t words = 0;
     size_t smem = 0;
@@ -124,8 +125,9 @@ struct JumpBatch {
 // generation kernel on a state array of its own with one row per launched
 // item (a whole stream, or one piece): `work` holds the items with their
 // rows in WorkItem::stream.  Before the kernel, `copies` (stream -> row)
-// give every row its stream's state and `jumps` advance the rows of pieces
-// after a stream's first by the piece's offset in the stream; after it,
+// give whole streams' and first pieces' rows their stream's state and the
+// jumps (jump_src -> jump_rows) give the rows of later pieces that state
+// advanced by the piece's offset in the stream; after it,
 // `backs` (row -> stream) return the state of every unsplit stream and of
 // every split stream's last piece.  row_set: parameter-set index of each
 // row's stream (handles with one set per stream).
@@ -138,7 +140,7 @@ struct SplitWork {
     std::vector<uint2> copies;
     std::vector<uint2> backs;
     std::vector<uint32_t> row_set;
-    std::vector<uint32_t> jump_rows, jump_sets;
+    std::vector<uint32_t> jump_rows, jump_src, jump_sets;
     std::vector<uint64_t> jump_lens;
 };
 
@@ -239,14 +241,19 @@ mtgp_status time_config(mtgp_streams* st, const Work& w, const LaunchCfg& cfg, u
 mtgp_status split_work(const Work& w, uint64_t max_piece, uint32_t max_pieces,
                        const std::vector<uint32_t>& set_of_stream, SplitWork* out);
 
-// Jump polynomials and items for advancing rows[i] (of the array the launch
-// is given) by jumps[i] numbers (0 = no jump); sets[i] = parameter set index.
+// Jump polynomials and items for giving rows[i] (of the array the launch
+// writes) the state of srcs[i] (of the array it reads) advanced by jumps[i]
+// numbers (0 = no jump); sets[i] = parameter set index.
 // host_sets: a host copy of the handle's per-stream parameter sets (null:
 // read from the device when needed).
 mtgp_status build_jump_batch(mtgp_streams* st, const std::vector<uint32_t>& rows,
-                             const std::vector<uint32_t>& sets, const std::vector<uint64_t>& jumps,
+                             const std::vector<uint32_t>& srcs, const std::vector<uint32_t>& sets, const std::vector<uint64_t>& jumps,
                              JumpBatch* out, const std::vector<KSet>* host_sets = nullptr);
-cudaError_t launch_jump_batch(const mtgp_streams* st, uint32_t* rows_base, const JumpItem* d_items,
+// Makes a few plain row copies items of the jump launch, so that no copy
+// kernel runs before it.
+void fold_copies(SplitWork* sw, JumpBatch* jb);
+cudaError_t launch_jump_batch(const mtgp_streams* st, const uint32_t* from, uint32_t* rows_base,
+                              const JumpItem* d_items,
                               uint32_t n, const uint32_t* d_polys, uint32_t words, size_t smem,
                               cudaStream_t s);
 

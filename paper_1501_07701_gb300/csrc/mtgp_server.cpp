@@ -262,12 +262,12 @@ extern "C" mtgp_status mtgp_server_create(mtgp_streams_t st, const mtgp_server_c
             } else {
                 // the jump polynomials of the piece offsets j * max_piece
                 // (j < 64) are computed once here rather than in a tick
-                std::vector<uint32_t> rows(63, 0u), sets(63, 0u);
+                const std::vector<uint32_t> rows(63, 0u), sets(63, 0u);
                 std::vector<uint64_t> lens(63);
                 for (uint32_t j = 0; j < 63u; ++j)
                     lens[j] = (uint64_t)(j + 1u) * c.max_piece;
                 JumpBatch jb;
-                mtgp_status r = build_jump_batch(st, rows, sets, lens, &jb);
+                mtgp_status r = build_jump_batch(st, rows, rows, sets, lens, &jb);
                 if (r != MTGP_OK) {
                     destroy_server(s);
                     return r;
@@ -416,6 +416,7 @@ static mtgp_status launch_split_tick(mtgp_server* s, Tick& t, const Work& w)
             const uint32_t j = (uint32_t)(sw.jump_lens[i] / s->cfg.max_piece) - 1u;
             JumpItem ji;
             ji.stream = sw.jump_rows[i];
+            ji.src = sw.jump_src[i];
             ji.poly = j;
             ji.deg = s->poly_deg[j];
             ji.set = 0;
@@ -424,11 +425,12 @@ static mtgp_status launch_split_tick(mtgp_server* s, Tick& t, const Work& w)
         jb.words = s->poly_words;
         jb.smem = s->jump_smem;
     } else {
-        r = build_jump_batch(st, sw.jump_rows, sw.jump_sets, sw.jump_lens, &jb,
+        r = build_jump_batch(st, sw.jump_rows, sw.jump_src, sw.jump_sets, sw.jump_lens, &jb,
                              st->d_sets ? &s->host_sets : nullptr);
         if (r != MTGP_OK)
             return r;
     }
+    fold_copies(&sw, &jb);
     const uint32_t N = st->P.k.n, np = st->P.k.np;
     const size_t rows_words = (size_t)sw.n_rows * np;
     if (rows_words > t.sp.rows_cap) {
@@ -469,7 +471,7 @@ static mtgp_status launch_split_tick(mtgp_server* s, Tick& t, const Work& w)
     CUDA_TRY_S(launch_copy_rows(st->d_states, t.sp.rows, (const uint2*)t.sp.aux, (uint32_t)sw.copies.size(),
                                 N, np, t.cs), "row copy");
     const uint32_t* polys = cached ? s->d_polys : (const uint32_t*)(t.sp.aux + o_poly);
-    CUDA_TRY_S(launch_jump_batch(st, t.sp.rows, (const JumpItem*)(t.sp.aux + o_ji), (uint32_t)jb.items.size(),
+    CUDA_TRY_S(launch_jump_batch(st, st->d_states, t.sp.rows, (const JumpItem*)(t.sp.aux + o_ji), (uint32_t)jb.items.size(),
                                  polys, jb.words, jb.smem, t.cs),
                "jump kernel");
     RowArray ra{t.sp.rows, sw.n_rows, st->d_sets ? (const uint32_t*)(t.sp.aux + o_set) : nullptr};
@@ -478,7 +480,7 @@ static mtgp_status launch_split_tick(mtgp_server* s, Tick& t, const Work& w)
         return r;
     CUDA_TRY_S(launch_copy_rows(t.sp.rows, st->d_states, (const uint2*)(t.sp.aux + o_backs),
                                 (uint32_t)sw.backs.size(), N, np, t.cs), "row copy back");
-    s->n_jumps += jb.items.size();
+    s->n_jumps += jb.items.size() - jb.n_copies;
     return MTGP_OK;
 }
 
