@@ -92,106 +92,40 @@ __device__ __forceinline__ void mt_sts(uint32_t a, uint32_t v)
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-template <int K, int FMT>
-__device__ __forceinline__ void mt_run_steps(const MtK& P, const MtSet& S, uint32_t* bp, uint32_t* op,
-                                             uint32_t nst, uint32_t lane);
-
-// Whole steps, by the loop that fits the set.
-template <int K, int FMT>
-__device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32_t* buf, uint32_t* op,
-                                            uint32_t nst, uint32_t lane);
-template <int K, int FMT>
-__device__ __forceinline__ void mt_run(const MtK& P, const MtSet& S, uint32_t* bp, uint32_t* op, uint32_t nst,
-                                       uint32_t lane)
-{
-    if (S.W == P.n - S.m)
-        mt_run_wide<K, FMT>(P, S, bp, op, nst, lane);
-    else
-        mt_run_steps<K, FMT>(P, S, bp, op, nst, lane);
-}
-
 // `nst` >= 1 whole steps inside one request, with room in the buffer for all
 // of them.  Lane j of sub-step i takes number k0 + 32 i + j of each step;
-// bp = buf + off + lane and op = the lane's output of the first step.
-// Lanes past W (32 K > W) load and compute too, on words of the buffer's
-// slack, so the step has no branches; only their two stores are predicated
-// off.  The tempering, conversion and output store of step t run after the
-// loads of step t + 1 are issued, so they fill the load latency instead of
-// lengthening the chain from one step's state store to the next step's loads.
-template <int K, int FMT>
-__device__ __forceinline__ void mt_run_steps(const MtK& P, const MtSet& S, uint32_t* bp, uint32_t* op,
-                                             uint32_t nst, uint32_t lane)
-{
-    const uint32_t W = S.W, m = S.m, n = P.n, upper = P.upper;
-    bool act[K];   // the lane's number in sub-step i belongs to the step
-#pragma unroll
-    for (int i = 0; i < K; ++i)
-        act[i] = 32u * i + lane < W;
-    uint32_t xn[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i)
-        xn[i] = mt_twist(upper, S, bp[32 * i], bp[32 * i + 1], bp[32 * i + m]);
-#pragma unroll
-    for (int i = 0; i < K; ++i)
-        if (act[i])
-            bp[32 * i + n] = xn[i];
-    __syncwarp();
-#pragma unroll 2
-    for (uint32_t t = 1; t < nst; ++t) {
-        bp += W;
-        uint32_t xt[K];
-#pragma unroll
-        for (int i = 0; i < K; ++i)
-            xt[i] = mt_twist(upper, S, bp[32 * i], bp[32 * i + 1], bp[32 * i + m]);
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            const uint32_t o = mt_convert<FMT>(mt_temper(S, xn[i]));
-            if (act[i])
-                __stcs(op + 32 * i, o);
-        }
-        op += W;
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            if (act[i])
-                bp[32 * i + n] = xt[i];
-            xn[i] = xt[i];
-        }
-        __syncwarp();
-    }
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-        const uint32_t o = mt_convert<FMT>(mt_temper(S, xn[i]));
-        if (act[i])
-            __stcs(op + 32 * i, o);
-    }
-}
-
-// The same for sets whose step is as wide as the recurrence allows, W = n - m
-// (n - m <= 256: the seed-generated sets up to n = 512, MT19937).
+// buf = the step's x_{k0} for this lane and op = the lane's output of the
+// first step.  The next step's loads fly while a step's numbers are
+// tempered, converted and stored; the chain from step to step is twist,
+// store, barrier and load.
 //
-// The middle word x_{k+W+m} of the next step's number is then the word x_{k+n}
-// that the same lane has just made, so it stays in a register: two shared
-// loads per number instead of three, and they fly while the step's numbers
-// are tempered, converted and stored.  The chain from step to step is twist,
-// store, barrier and load.  Lanes past W store too, behind the step's words
-// (in the buffer's slack at its end): only words of later steps come there,
-// each stored before it is read.
+// OWN: the step is as wide as the recurrence allows, W = n - m (n - m <= 256:
+// the seed-generated sets up to n = 512, MT19937).  The middle word x_{k+W+m}
+// of the next step's number is then the word x_{k+n} that the same lane has
+// just made, so it stays in a register: two shared loads per number instead
+// of three.
+//
+// Lanes past W load and compute too, on words of the buffer's slack, so the
+// step has no branches; only their output is predicated off.  They store too,
+// behind the step's words (in the buffer's slack at its end): only words of
+// later steps come there, each stored before it is read.
 // What bounds it: that chain, 130 cycles per step for a warp alone and 172 for
-// two warps per SM quarter (p = 3217, 51 numbers per step).  Measured: the
-// uneven 10 000-stream workload 7.80 -> 6.85 ms at p = 3217 and 6.94 -> 6.06 ms
-// for MT19937.  Reading a whole step ahead, with the one or two words it then
-// lacks at p = 3217 by shuffle, took more instructions than it hid latency
-// (9.6 ms).
-template <int K, int FMT>
-__device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32_t* buf, uint32_t* op,
-                                            uint32_t nst, uint32_t lane)
+// two warps per SM quarter (p = 3217, 51 numbers per step).  Measured, uneven
+// 10 000-stream workload, against the loop that loaded all three words first
+// and tempered the previous step after: p = 3217 7.70 -> 6.97 ms, MT19937 7.16
+// -> 5.93, p = 44497 7.32 -> 6.33.  Reading a whole step ahead, with the one or
+// two words it then lacks at p = 3217 by shuffle, took more instructions than
+// it hid latency (9.6 ms).
+template <int K, int FMT, bool OWN>
+__device__ __forceinline__ void mt_run_steps(const MtK& P, const MtSet& S, uint32_t* buf, uint32_t* op,
+                                             uint32_t nst, uint32_t lane)
 {
     const uint32_t W = S.W, upper = P.upper;
     const uint32_t step = 4u * W;
     uint32_t rd = (uint32_t)__cvta_generic_to_shared(buf);   // this lane's x_k
     uint32_t wr = rd + 4u * P.n;                             // and x_{k+n}
     bool act[K];
-    uint32_t x0[K], x1[K], xm[K];
+    uint32_t x0[K], x1[K], x2[K], xm[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
         act[i] = 32u * i + lane < W;
@@ -199,8 +133,7 @@ __device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32
         x1[i] = mt_lds(rd + 128u * i + 4u);
         xm[i] = mt_lds(rd + 128u * i + 4u * S.m);
     }
-    constexpr int U = K == 4 ? 4 : 2;   // as measured per step width
-#pragma unroll U
+#pragma unroll 6
     for (uint32_t t = 0; t < nst; ++t) {
 #pragma unroll
         for (int i = 0; i < K; ++i)
@@ -215,11 +148,16 @@ __device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32
         for (int i = 0; i < K; ++i) {
             x0[i] = mt_lds(rd + 128u * i);
             x1[i] = mt_lds(rd + 128u * i + 4u);
+            if (!OWN)
+                x2[i] = mt_lds(rd + 128u * i + 4u * S.m);
         }
         uint32_t o[K];
 #pragma unroll
-        for (int i = 0; i < K; ++i)
+        for (int i = 0; i < K; ++i) {
             o[i] = mt_convert<FMT>(mt_temper(S, xm[i]));
+            if (!OWN)
+                xm[i] = x2[i];
+        }
 #pragma unroll
         for (int i = 0; i < K; ++i)
             asm volatile("" : "+r"(o[i]));   // not moved under the store's condition
@@ -230,6 +168,16 @@ __device__ __forceinline__ void mt_run_wide(const MtK& P, const MtSet& S, uint32
         op += W;
     }
     __syncwarp();   // the loads above come before the buffer's next writes
+}
+
+template <int K, int FMT>
+__device__ __forceinline__ void mt_run(const MtK& P, const MtSet& S, uint32_t* bp, uint32_t* op, uint32_t nst,
+                                       uint32_t lane)
+{
+    if (S.W == P.n - S.m)
+        mt_run_steps<K, FMT, true>(P, S, bp, op, nst, lane);
+    else
+        mt_run_steps<K, FMT, false>(P, S, bp, op, nst, lane);
 }
 
 // A step that crosses a request boundary or the stream's end: each lane finds
@@ -263,8 +211,10 @@ __device__ __forceinline__ void mt_step_slow(const MtK& P, const MtSet& S, uint3
     }
 }
 
+// (The bound of 16 warps per SM, 128 registers, is for the step loop: left to
+// itself the compiler took half of them and the loop ran 5 to 20 % slower.)
 template <int K>
-__global__ void __launch_bounds__(128) mt_gen_kernel(const MtK P, uint32_t* __restrict__ states,
+__global__ void __launch_bounds__(128, 4) mt_gen_kernel(const MtK P, uint32_t* __restrict__ states,
                                                      uint32_t n_streams,
                                                      const WorkItem* __restrict__ items,
                                                      const Segment* __restrict__ segs,
