@@ -15,11 +15,12 @@
 //   * Column group m (columns 32m .. 32m+31) belongs to one warp; lane l of
 //     that warp keeps column 32m + l in a register (word i).
 //   * The latest value of every column is also published in a shared-memory
-//     row S[0..N), followed by a mirror S[N..N+E) of columns 0..E-1,
-//     E >= pos + 31.  Words i+1, i+pos and i+pos-1 of 32 consecutive columns
-//     are then plain conflict-free loads at S[c+1], S[c+pos], S[c+pos-1]
-//     with no modulo and no bounds arithmetic: a pick-up past column N-1
-//     lands in the mirror, which holds the new row's value of that column.
+//     row S[0..N), where words i+1 and i+pos of 32 consecutive columns are
+//     plain conflict-free loads.  A pick-up past column N-1 is the new row's
+//     value of column c+pos-N: the late-tempering loops keep each group's
+//     pick-up address with that wrap in it; the other loops (CTA-wide
+//     streams, K = 8, N - pos < 256) mirror columns 0..E-1, E >= pos + 31,
+//     at S[N..N+E), so that S[c+1], S[c+pos] and S[c+pos-1] need no wrap.
 //   * The recursion and tempering tables are 16-word shared arrays whose entry
 //     k sits in bank k, so a warp's 32 lookups are one conflict-free
 //     shared-memory wavefront whatever the indices.
