@@ -1604,11 +1604,12 @@ static mtgp_status build_split_stats(mtgp_plan* p)
 
 // Kernel and launch geometry of a plan's fused statistics: G = 8 warps per
 // CTA, as many resident CTAs per SM as the plan's configuration asks warps
-// per SM (warps_per_cta x ctas_per_sm / 8, at least 1; occupancy maximum when
-// ctas_per_sm is 0), persistent grid.  The kernel takes single-warp items
-// with 128-word pipelined steps, so every parameter set needs N - pos >= 256,
-// or N - pos >= 32 for short states (ceil(N/32) < 9); the handle's
-// representative set has the largest pos of its sets.
+// per SM (warps_per_cta x ctas_per_sm / 8, at least 1, rounded up for an
+// automatic shape; occupancy maximum when ctas_per_sm is 0), persistent
+// grid.  The kernel takes single-warp items with 128-word pipelined steps, so
+// every parameter set needs N - pos >= 256, or N - pos >= 32 for short states
+// (ceil(N/32) < 9); the handle's representative set has the largest pos of
+// its sets.
 static mtgp_status stats_geometry(mtgp_plan* p)
 {
     mtgp_streams* st = p->st;
@@ -1633,8 +1634,12 @@ static mtgp_status stats_geometry(mtgp_plan* p)
              "statistics kernel occupancy");
     if (per_sm < 1)
         return fail(MTGP_EINVAL, "statistics kernel does not fit on an SM");
+    // an automatic shape of 12 warps (no stream longer than a warp's share
+    // there) rounds up: the statistics' latency takes 16 warps to hide
+    // (2432 x 2^19, Mexp 23209: 1.94 ms on 16 warps per SM, 2.80 on 8)
+    const int warps = p->cfg.warps_per_cta * p->cfg.ctas_per_sm + (p->cfg.automatic ? G - 1 : 0);
     if (p->cfg.ctas_per_sm > 0)
-        per_sm = std::min(per_sm, std::max(1, p->cfg.warps_per_cta * p->cfg.ctas_per_sm / G));
+        per_sm = std::min(per_sm, std::max(1, warps / G));
     cudaFuncAttributes fa;
     CUDA_TRY(cudaFuncGetAttributes(&fa, fn), "cudaFuncGetAttributes");
     int sms = 0;

@@ -324,8 +324,8 @@ __device__ __forceinline__ void ham_step(const uint32_t (&w)[4], uint32_t step_n
 // of the loop.  Measured (one launch, 5.12 G numbers, Mexp 11213): 14.0 -> 10.6
 // ms at 8 warps per SM, 10.3 -> 7.35 ms at 16 split in pieces of 1 052 897;
 // 2432 x 2^19 at Mexp 23209 and 16 warps per SM 2.44 -> 1.94 ms, at Mexp 44497
-// and 8 3.61 -> 2.53 ms (its registers leave no room for 16).  What bounds it:
-// issue and latency, about 165 instructions per 128 numbers.
+// 2.55 -> 2.24 ms.  What bounds it: issue and latency, about 165 instructions
+// per 128 numbers.
 template <int M, int FMT, bool STEPH>
 __device__ __forceinline__ void fused_rows(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
                                            const uint32_t* __restrict__ Tb, uint32_t nfull, StatsState& st,
@@ -663,9 +663,12 @@ __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uin
 }
 
 // Persistent kernel: every warp claims streams (longest first) from the
-// work table and advances each alone, with the statistics.
+// work table and advances each alone, with the statistics.  Bounded to 128
+// registers, for 16 warps per SM, also where that spills (M = 44: 450 loads in
+// the whole kernel): 2432 x 2^19 at Mexp 44497 takes 2.24 ms at 16 warps, and
+// 2.53 at the 8 that its 255 registers would leave room for.
 template <int M, int G>
-__global__ void __launch_bounds__(G * 32, M < 32 ? 2 : 1) mtgp_fused_kernel(const KParams P, uint32_t* __restrict__ states,
+__global__ void __launch_bounds__(G * 32, 2) mtgp_fused_kernel(const KParams P, uint32_t* __restrict__ states,
                                                             uint32_t n_streams,
                                                             const WorkItem* __restrict__ items,
                                                             const Segment* __restrict__ segs,
