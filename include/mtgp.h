@@ -256,8 +256,8 @@ mtgp_status mtgp_autotune(mtgp_streams_t streams, mtgp_format fmt, uint32_t samp
  * mtgp_generate_u32; every request in format `fmt`; `out` is a device
  * pointer that must stay valid while the plan is used).  The work table is
  * sorted longest stream first and uploaded once; launching replays a CUDA
- * graph (reset of the work counter + one persistent kernel whose warps claim
- * streams from that table).  The plan keeps a reference to `streams`. */
+ * graph (reset of the claim counters, where they are used, + one persistent
+ * kernel whose warps claim streams from that table).  The plan keeps a reference to `streams`. */
 mtgp_status mtgp_plan_create(mtgp_streams_t streams, const uint32_t* stream_ids,
                              const uint64_t* counts, uint32_t n_req, mtgp_format fmt,
                              void* out, mtgp_plan_t* plan);
