@@ -266,7 +266,10 @@ __device__ __forceinline__ void gen_row(uint32_t (&r)[(M + WG - 1) / WG], uint32
 // N-1 is column 0 of the new row (`x1_last` points there): written in step 0
 // and read in step NS-2 >= 1 or later.  The loads issued during a row's last
 // step are those of step 0 (the same addresses in every row); after the last
-// row they are simply unused.  Lanes past column N-1 in the last group
+// row they are simply unused.  Before the first row these loads are made apart,
+// and the numbers after the loop read neighbours' words too, which a run that
+// follows at once (a request that ends with a row) overwrites in its step 0: a
+// barrier before the loop orders both before step 0's stores.  Lanes past column N-1 in the last group
 // compute on the words behind the row and write there; only their output
 // store is predicated off.
 //
@@ -370,6 +373,7 @@ __device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const R
         x1[i] = lds_at<128 * i + 4>(sa);
         xp[i] = lds_at<0>(qa[i]);
     });
+    __syncwarp();   // these loads, and the last ones of a run before, come before step 0's stores
     uint32_t* op = ow + 1 - (int)N;   // where column `lane` of this row stores
 #pragma unroll U
     for (uint32_t q = 0; q < nfull; ++q, op += N) {
@@ -469,6 +473,7 @@ __device__ __forceinline__ void gen_rows_short(uint32_t* S, uint32_t* ow, const 
     static_for<4 * NT>([&](auto i) { xs[i.value] = 0u; });
     T[NT - 1] = (temper_index(S[P.pos - 1u]) & 15u) << (2 + 8 * ((M - 1) & 3));
     uint32_t x1 = lds_at<4>(sa), xp = lds_at<0>(qa[0]);
+    __syncwarp();   // as in gen_rows_late
     uint32_t* op = ow + 1 - (int)N;
 #pragma unroll 4
     for (uint32_t q = 0; q < nfull; ++q, op += N) {

@@ -359,6 +359,7 @@ __device__ __forceinline__ void fused_rows(uint32_t* S, uint32_t* ow, const RowP
         x1[i] = lds_at<128 * i + 4>(sa);
         xp[i] = lds_at<0>(qa[i]);
     });
+    __syncwarp();   // before step 0's stores, as in gen_rows_late
     uint32_t* op = ow + 1 - (int)N;
     // the gap window: this lane's ballot, its place in the window, rows in it
     uint32_t vw = 0u, rb = 0u, slot = lane;   // slot: lane less the window's earlier groups
@@ -498,6 +499,7 @@ __device__ __forceinline__ void fused_rows_short(uint32_t* S, uint32_t* ow, cons
     uint32_t x1 = Sw[1];
     uint32_t xp = *Qp[0];
     uint32_t xq = *Qq[0];
+    __syncwarp();   // these loads come before the first sub-step's stores
     for (uint32_t q = 0; q < nfull; ++q, ow += N) {
 #pragma unroll
         for (int m = 0; m < M; ++m) {
