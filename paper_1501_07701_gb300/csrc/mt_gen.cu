@@ -613,6 +613,25 @@ extern "C" mtgp_status mtgp_mt_get_statuses(mtgp_mt_t h, uint32_t* states, void*
     return ok();
 }
 
+// CTAs of a launch over `n_items` >= 1 streams, `total` numbers in all and
+// `max_item` in the longest.  Every stream runs on one warp, longest first, so
+// the launch cannot end before its longest stream does.  About total / longest
+// warps keep pace with that stream; more warps only slow it down by sharing its
+// SM.  At least one CTA per SM.
+// A few CTAs over a whole number per SM would slow those SMs' streams, so they
+// are left out where streams outnumber the warps and the others take their
+// share (uneven workload, 306 CTAs to 304).  Never where every stream would
+// have had a warp: 612 to 684 equal streams of 2^16 at p = 3217 take 0.20 ms on
+// 152 CTAs, a second round for a few of them, and 0.147 with the CTAs kept.
+static long long mt_ctas(uint32_t n_items, uint64_t total, uint64_t max_item, int sms)
+{
+    const long long pace = (long long)((total + max_item - 1) / max_item);
+    const long long warps = std::max<long long>(pace, (long long)sms * kWarpsPerCta);
+    const long long want = (std::min<long long>(n_items, warps) + kWarpsPerCta - 1) / kWarpsPerCta;
+    const long long over = want > sms ? want % sms : 0;
+    return over <= sms / 8 && n_items >= 2 * want * kWarpsPerCta ? want - over : want;
+}
+
 extern "C" mtgp_status mtgp_mt_generate(mtgp_mt_t h, const uint32_t* ids, const uint64_t* counts,
                                         uint32_t n_req, mtgp_format fmt, void* out, void* cuda_stream)
 {
@@ -654,17 +673,8 @@ extern "C" mtgp_status mtgp_mt_generate(mtgp_mt_t h, const uint32_t* ids, const 
         fill_table(w, sl.host);
         MT_TRY(cudaMemcpyAsync(sl.dev, sl.host, bytes, cudaMemcpyHostToDevice, s),
                "cudaMemcpyAsync(work table)");
-        // Warp count: every stream runs on one warp, longest first, so the
-        // launch cannot end before its longest stream does.  About
-        // total / longest warps keep pace with that stream; more warps only
-        // slow it down by sharing its SM.  At least one CTA per SM.
         const uint32_t n_items = (uint32_t)w.items.size();
-        const long long pace = (long long)((w.total + w.max_item - 1) / w.max_item);
-        const long long warps = std::max<long long>(pace, (long long)h->sms * kWarpsPerCta);
-        long long want = (std::min<long long>(n_items, warps) + kWarpsPerCta - 1) / kWarpsPerCta;
-        // a few CTAs over a whole number per SM would slow those SMs' streams
-        if (want > h->sms && want % h->sms <= h->sms / 8)
-            want -= want % h->sms;
+        const long long want = mt_ctas(n_items, w.total, w.max_item, h->sms);
         const int grid = (int)std::max(1LL, std::min<long long>(want, h->grid_cap));
         const WorkItem* items = (const WorkItem*)((char*)sl.dev + io);
         const Segment* segs = (const Segment*)((char*)sl.dev + so);
