@@ -198,15 +198,16 @@ mtgp_status mtgp_generate_to_host(mtgp_streams_t streams, const uint32_t* stream
  * no cudaMalloc, cudaFree or other allocating routine: the work table lives
  * in a 64 KiB statically declared device array that every device loading the
  * library holds until exit.  The first call on a device looks that array's
- * address up (cudaGetSymbolAddress); make that first call before any stream
- * capture.  All calls on a device share the array and each overwrites the
- * previous contents (the claim counters are cleared on every call), so calls
- * whose kernels overlap on the GPU race: order them (one CUDA stream, one
- * host thread at a time).  The work table is copied from a host array that
- * the next call overwrites, so a call made while cuda_stream is being
- * captured returns MTGP_EINVAL (record graphs with mtgp_plan_create).  The
- * array's address is looked up once per device for the life of the
- * process: a cudaDeviceReset while the library is loaded is not supported
+ * address up (cudaGetSymbolAddress), and the first on a handle the launch
+ * shapes of all sizes; make that first call before any stream capture.
+ * All calls on a device share the array and each overwrites the previous
+ * contents (the claim counters are cleared on every call), so calls whose
+ * kernels overlap on the GPU race: order them (one CUDA stream, one host
+ * thread at a time).  The work table is copied from a host array that the
+ * next call overwrites, so a call made while cuda_stream is being captured
+ * returns MTGP_EINVAL (record graphs with mtgp_plan_create).  The array's
+ * address is looked up once per device for the life of the process: a
+ * cudaDeviceReset while the library is loaded is not supported
  * by this call.  Asynchronous on cuda_stream. */
 mtgp_status mtgp_generate_noalloc(mtgp_streams_t streams, const uint32_t* stream_ids,
                                   const uint64_t* counts, uint32_t n_req, mtgp_format fmt,

@@ -809,19 +809,36 @@ extern "C" mtgp_status mtgp_get_statuses(mtgp_streams_t st, uint32_t* states, vo
     GUARD_END
 }
 
-// Resolves the geometry for the handle's configuration (cached).
+// Resolves the geometry of a configuration (cached in the handle, without heap
+// memory: the calls that must not enter the allocator come here too).
 mtgp_status mtgp::geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, Geometry* g)
 {
     const auto key = std::make_tuple(cfg.warps_per_cta, cfg.ctas_per_sm, cfg.k, cfg.kernel);
-    auto it = st->geo_caps.find(key);
-    if (it == st->geo_caps.end()) {
-        Geometry full;
-        cudaError_t e = plan_geometry(st->P.k, cfg, 0x7FFFFFFF, st->device, &full);
-        if (e != cudaSuccess)
-            return fail_cuda(e, "launch geometry");
-        it = st->geo_caps.emplace(key, full).first;
+    int at = -1;
+    if (cfg.automatic) {
+        for (int i = 0; i < kNumAutoShapes; ++i)
+            if (kAutoShapes[i].warps_per_cta == cfg.warps_per_cta && kAutoShapes[i].ctas_per_sm == cfg.ctas_per_sm)
+                at = i;
+    } else {
+        for (int i = kNumAutoShapes; i < (int)st->geos.size(); ++i)
+            if (st->geos[i].valid && st->geos[i].key == key)
+                at = i;
     }
-    *g = it->second;
+    if (at < 0 || !st->geos[at].valid || st->geos[at].key != key) {
+        GeoEntry e;
+        e.key = key;
+        cudaError_t err = plan_geometry(st->P.k, cfg, 0x7FFFFFFF, st->device, &e.g);
+        if (err != cudaSuccess)
+            return fail_cuda(err, "launch geometry");
+        e.valid = true;
+        if (at < 0) {
+            at = kNumAutoShapes + st->next_geo;
+            st->next_geo = (st->next_geo + 1) % mtgp_streams::kExplicitGeos;
+        }
+        st->geos[at] = e;
+    }
+    const Geometry& full = st->geos[at].g;
+    *g = full;
     // One CTA per item at most (a CTA may take a whole stream), and without
     // CTA-wide streams no more CTAs per SM than give every item a warp.
     const long long items = (long long)n_items;
@@ -830,8 +847,22 @@ mtgp_status mtgp::geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t 
         const long long slots = (long long)st->sms * (g->threads / 32);
         want = std::min<long long>(want, st->sms * ((items + slots - 1) / slots));
     }
-    g->grid = (int)std::max(1LL, std::min<long long>(want, it->second.grid));
+    g->grid = (int)std::max(1LL, std::min<long long>(want, full.grid));
     return MTGP_OK;
+}
+
+void mtgp::resolve_shapes(mtgp_streams* st)
+{
+    if (!st->cfg.automatic || st->shapes_resolved)   // explicit: one configuration for all sizes
+        return;
+    Geometry g;
+    for (const AutoShape& sh : kAutoShapes) {
+        LaunchCfg c = st->cfg;
+        c.warps_per_cta = sh.warps_per_cta;
+        c.ctas_per_sm = sh.ctas_per_sm;
+        geometry_for(st, c, 1, &g);   // one that cannot launch is reported when a call chooses it
+    }
+    st->shapes_resolved = true;
 }
 
 // Uploads a work table through the handle's slot ring and launches.

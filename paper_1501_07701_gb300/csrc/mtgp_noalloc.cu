@@ -33,7 +33,7 @@ using namespace mtgp;
 
 namespace {
 
-// Largest request list one call accepts.  The table holds the two claim
+// Largest request list one call accepts.  The table holds the claim
 // counters (kCounterBytes, cleared on every call), one 16-byte item per
 // distinct stream and one 32-byte segment per request.
 constexpr uint32_t kMaxRequests = 1024;
@@ -178,6 +178,9 @@ extern "C" mtgp_status mtgp_generate_noalloc(mtgp_streams_t st, const uint32_t* 
         T.item_total[b] = tt;
     }
 
+    // The first call looks all of the handle's launch shapes up: a later call
+    // of another size then makes no queries.
+    resolve_shapes(st);
     Geometry g;
     const LaunchCfg run = fit_config(st, st->cfg, n_items, total, T.item_total[0]);
     mtgp_status s = geometry_for(st, run, n_items, &g);

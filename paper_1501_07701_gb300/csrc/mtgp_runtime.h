@@ -3,7 +3,6 @@
 #pragma once
 
 #include <array>
-#include <map>
 #include <new>
 #include <tuple>
 #include <vector>
@@ -36,6 +35,21 @@ struct BuildScratch {
     std::vector<uint64_t> off, keys;
     std::vector<WorkItem> sorted;
     std::vector<uint64_t> tot;
+};
+
+// Launch shapes that fit_config chooses among.
+struct AutoShape {
+    int warps_per_cta;
+    int ctas_per_sm;
+};
+constexpr AutoShape kAutoShapes[] = {{4, 1}, {4, 2}, {4, 3}, {8, 1}, {8, 2}};
+constexpr int kNumAutoShapes = (int)(sizeof kAutoShapes / sizeof kAutoShapes[0]);
+
+// Geometry of one configuration (warps per CTA, CTAs per SM, sub-steps, kernel).
+struct GeoEntry {
+    bool valid = false;
+    std::tuple<int, int, int, int> key{};
+    Geometry g{};
 };
 
 // A pinned host buffer and a device buffer holding one uploaded work table
@@ -84,9 +98,12 @@ struct mtgp_streams {
     mtgp::LaunchCfg cfg{};
     std::array<mtgp::TableSlot, 4> slots{};
     int next_slot = 0;
-    // launch geometry per configuration (warps per CTA, CTAs per SM, sub-steps,
-    // kernel; grid = residency cap)
-    std::map<std::tuple<int, int, int, int>, mtgp::Geometry> geo_caps;
+    // launch geometry per configuration (grid = residency cap): the automatic
+    // shapes at their places, then the explicit configurations last used
+    static constexpr int kExplicitGeos = 4;
+    std::array<mtgp::GeoEntry, mtgp::kNumAutoShapes + kExplicitGeos> geos{};
+    int next_geo = 0;
+    bool shapes_resolved = false;
     // device-to-host path
     // (kStages buffers: generation may run that many chunks ahead of the copies)
     static constexpr int kStages = 4;
@@ -207,6 +224,9 @@ LaunchCfg default_config(const KParams& P);
 LaunchCfg fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
                      uint64_t max_item);
 mtgp_status geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, Geometry* g);
+// Resolves the geometry of every shape that fit_config may choose for the
+// handle's configuration, so that later calls of any size look none up.
+void resolve_shapes(mtgp_streams* st);
 mtgp_status launch_work(mtgp_streams* st, const Work& w, const LaunchCfg& cfg, void* out,
                         cudaStream_t s);
 // A launch's own state rows (a split launch: one row per item, see
