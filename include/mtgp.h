@@ -236,9 +236,18 @@ typedef struct {
                                  1 = shared-memory ring path (any parameters)  */
     uint32_t coop_percent;    /* streams of a launch longer than coop_percent/100
                                  times the numbers per warp slot are advanced
-                                 by a whole CTA (longest first); 0 = never     */
+                                 by a whole CTA (longest first); 0 = never.
+                                 Needs words_per_lane >= warps_per_cta and one
+                                 parameter set, else no stream is             */
 } mtgp_launch_config;
 
+/* The configuration of the handle's launches.  A new handle has the default:
+ * warps_per_cta 4, ctas_per_sm 2, coop_percent 0 and words_per_lane by the
+ * parameter set.  These values stand for a launch shape that the library
+ * chooses for each launch by its number of streams and their lengths (the
+ * ring path runs them as they are); setting them returns a handle to that.
+ * Any other configuration is used as given.  mtgp_plan_get_info reports the
+ * shape that a plan runs with. */
 mtgp_status mtgp_get_launch_config(mtgp_streams_t streams, mtgp_launch_config* cfg);
 mtgp_status mtgp_set_launch_config(mtgp_streams_t streams, const mtgp_launch_config* cfg);
 

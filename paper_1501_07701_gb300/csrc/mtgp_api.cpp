@@ -697,23 +697,30 @@ extern "C" mtgp_status mtgp_init_statuses_multi(const mtgp_params_t* sets, uint3
 
 LaunchCfg mtgp::default_config(const KParams& P)
 {
-    // 8 warps per SM, in one CTA; 128-word software-pipelined steps when the parameter
-    // set allows them (N - pos >= 256), else 256-word steps, else 128, else
-    // 64 (short states such as Mexp 3217).
+    // 8 warps per SM in 4-warp CTAs; 128-word software-pipelined steps when the
+    // parameter set allows them (N - pos >= 256), else 256-word steps, else
+    // 128, else 64 (short states such as Mexp 3217).
     LaunchCfg c;
-    c.warps_per_cta = 8;
-    c.ctas_per_sm = 1;
+    c.warps_per_cta = 4;
+    c.ctas_per_sm = 2;
     c.k = 4;
     c.kernel = 0;
     c.coop_percent = 0;
     if (P.n - P.pos < 256u || !fast_supported(P, 4))
         c.k = fast_supported(P, 8) ? 8 : (fast_supported(P, 4) || !fast_supported(P, 2) ? 4 : 2);
+    // fit_config chooses the shape of each launch (not for the ring kernel)
     c.automatic = fast_supported(P, c.k, 8) && fast_supported(P, c.k, 4);
-    if (!c.automatic) {   // the ring kernel: large states leave room for four warps per CTA
-        c.warps_per_cta = 4;
-        c.ctas_per_sm = 2;
-    }
     return c;
+}
+
+// These values stand for the default wherever they come from, so that a
+// configuration that was read can be set again, on this handle or another.
+LaunchCfg mtgp::recognise_default(const KParams& P, const LaunchCfg& c)
+{
+    const LaunchCfg d = default_config(P);
+    const bool same = c.warps_per_cta == d.warps_per_cta && c.ctas_per_sm == d.ctas_per_sm && c.k == d.k &&
+                      c.kernel == d.kernel && c.coop_percent == d.coop_percent;
+    return same ? d : c;
 }
 
 LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
@@ -1213,7 +1220,7 @@ extern "C" mtgp_status mtgp_set_launch_config(mtgp_streams_t st, const mtgp_laun
     mtgp_status s = validate_config(cfg, &c);
     if (s != MTGP_OK)
         return s;
-    st->cfg = c;
+    st->cfg = recognise_default(st->P.k, c);
     return ok();
 }
 
@@ -1236,7 +1243,7 @@ std::vector<LaunchCfg> mtgp::tuning_candidates(const KParams& P)
         x.kernel = 0;
         x.coop_percent = coop;
         x.automatic = false;
-        v.push_back(x);
+        v.push_back(recognise_default(P, x));
     };
     for (int k : {8, 4, 2}) {
         for (int cap : {1, 2, 3, 4, 0})
@@ -1819,7 +1826,7 @@ extern "C" mtgp_status mtgp_plan_autotune(mtgp_plan_t p, mtgp_launch_config* bes
     cudaFree(scratch);
     if (r != MTGP_OK)
         return r;
-    p->cfg = win;
+    p->cfg = fit_config(st, win, p->n_items, p->split.work.total, p->max_item);
     r = geometry_for(st, p->cfg, p->n_items, &p->geo);
     if (r != MTGP_OK)
         return r;

@@ -218,6 +218,8 @@ mtgp_status build_work(uint32_t n_streams, const uint32_t* ids, const uint64_t* 
 size_t table_bytes(const Work& w, size_t* items_off, size_t* segs_off);
 void fill_table(const Work& w, void* host);
 LaunchCfg default_config(const KParams& P);
+// `c`, or the default configuration if `c` has its values.
+LaunchCfg recognise_default(const KParams& P, const LaunchCfg& c);
 // The configuration a launch of this work runs with: `cfg` itself, or for the
 // default configuration its warps per CTA and CTAs per SM chosen from the
 // number of items, their total and the longest.
