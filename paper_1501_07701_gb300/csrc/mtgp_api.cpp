@@ -906,8 +906,14 @@ mtgp_status mtgp::reserve_slot(TableSlot& sl, size_t bytes)
 }
 
 // Largest work table (bytes after the counters) that a launch reads from host
-// memory.
+// memory, and the most requests one of its streams may have.  A row that
+// crosses requests has every lane walk the stream's list, one dependent read
+// after the other, so long lists are copied: 16 requests of one stream take 72
+// us from device memory and 77 read in place, 500 take 548 and 795; up to 4 a
+// stream the copy's own 2 to 4 us are the larger part (400 requests, 4 a
+// stream: 44.6 copied, 42.0 in place).
 static constexpr size_t kInPlaceTable = 16384;
+static constexpr uint32_t kInPlaceRequests = 4;
 
 // Hands a work table to a launch through `sl` (waiting for the slot's previous
 // consumer) and launches on `s`; records the slot's event after the kernel.
@@ -927,11 +933,14 @@ mtgp_status mtgp::launch_work_slot(mtgp_streams* st, TableSlot& sl, const Work& 
     r = geometry_for(st, run, (uint32_t)w.items.size(), &g);
     if (r != MTGP_OK)
         return r;
-    // A launch whose items are placed reads each entry of the table once and
-    // needs no counters, so a small table stays in the pinned host buffer and
-    // the warps read it there: no copy for the kernel to wait for.
+    // A launch whose items are placed needs no counters and, where streams have
+    // few requests, reads each entry of the table about once, so a small table
+    // stays in the pinned host buffer and the warps read it there: no copy for
+    // the kernel to wait for.
     const bool in_place = bytes <= kCounterBytes + kInPlaceTable && g.kernel == 0 && run.coop_percent == 0 &&
-                          items_placed((uint32_t)w.items.size(), (uint32_t)g.grid, (uint32_t)g.threads / 32u);
+                          items_placed((uint32_t)w.items.size(), (uint32_t)g.grid, (uint32_t)g.threads / 32u) &&
+                          std::all_of(w.items.begin(), w.items.end(),
+                                      [](const WorkItem& it) { return it.nseg <= kInPlaceRequests; });
     if (!in_place)
         CUDA_TRY(cudaMemcpyAsync(sl.dev, sl.host, bytes, cudaMemcpyHostToDevice, s),
                  "cudaMemcpyAsync(work table)");
