@@ -978,6 +978,7 @@ mtgp_status mtgp::launch_work_table(mtgp_streams* st, const Work& w, void* table
     a.trace = nullptr;
     a.sets = st->d_sets;
     a.set_of = st->d_set_of;
+    a.one_list = one_claim_list(w.max_item);
     if (rows) {
         a.states = rows->states;
         a.n_streams = rows->n_rows;
@@ -1453,6 +1454,7 @@ static mtgp_status record_graph(mtgp_plan* p)
     a.trace = p->d_trace;
     a.sets = p->st->d_sets;
     a.set_of = split ? p->d_row_set : p->st->d_set_of;
+    a.one_list = one_claim_list(p->max_item);
     const bool counted = p->stats || p->geo.kernel != 0 || a.n_coop ||
                          !items_placed(p->n_items, (uint32_t)p->geo.grid, (uint32_t)p->geo.threads / 32u);
     if (e1 == cudaSuccess && counted)

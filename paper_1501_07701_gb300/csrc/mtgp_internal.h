@@ -111,6 +111,15 @@ __host__ __device__ inline bool items_placed(uint32_t n_items, uint32_t grid, ui
     return (uint64_t)n_items <= (uint64_t)grid * warps;
 }
 
+// True if a launch claims its items from one list instead of one per SM.
+// Lists per SM share long streams out evenly, but a warp that finds its own
+// list used up reads all the others' counters: 3 to 6 us at a launch's end,
+// against the 10 us that a stream of 2^14 numbers takes.  One list against one
+// per SM: 10 000 streams of 2^2 .. 2^8 numbers 20.7 and 25.4 us at Mexp 11213,
+// 27.3 and 30.8 at 23209; 2538 of 2^7 .. 2^14 22.9 and 24.9, 24.5 and 27.3;
+// 2538 of 2^9 .. 2^16, in the automatic shape, 63.5 and 52.6, 66.8 and 59.2.
+inline bool one_claim_list(uint64_t max_item) { return max_item <= (1u << 14); }
+
 struct GenArgs {
     KParams P;
     uint32_t* states;
@@ -125,6 +134,7 @@ struct GenArgs {
     uint64_t* trace;     // optional: 4 words per item (start ns, end ns, SM, numbers)
     const KSet* sets = nullptr;        // per-stream parameter sets (null: every stream uses P)
     const uint32_t* set_of = nullptr;  // set index of each stream when `sets` is given
+    bool one_list = false;             // items are claimed from one list (see one_claim_list)
 };
 
 // Jump of one state row by a count J: from row `src` of the array a launch

@@ -361,7 +361,7 @@ cudaError_t launch_gen_fn(const void* fn, const GenArgs& a, dim3 grid, dim3 bloc
     uint64_t* trace = a.trace;
     const KSet* sets = a.sets;
     const uint32_t* set_of = a.set_of;
-    uint32_t n_groups = std::max(1u, std::min(std::min(grid.x, sms), kMaxGroups));
+    uint32_t n_groups = a.one_list ? 1u : std::max(1u, std::min(std::min(grid.x, sms), kMaxGroups));
     void* args[] = {&P, &states, &n_streams, &items, &segs, &n_items, &n_coop, &counter, &out, &err,
                     &trace, &sets, &set_of, &n_groups};
     return cudaLaunchKernel(fn, grid, block, args, smem, s);

@@ -216,6 +216,7 @@ extern "C" mtgp_status mtgp_generate_noalloc(mtgp_streams_t st, const uint32_t* 
     a.trace = nullptr;
     a.sets = st->d_sets;
     a.set_of = st->d_set_of;
+    a.one_list = one_claim_list(T.item_total[0]);
     e = launch_generate(a, g, cs);
     if (e != cudaSuccess)
         return fail_cuda(e, "generation kernel launch (no-alloc)");
