@@ -723,12 +723,11 @@ LaunchCfg mtgp::recognise_default(const KParams& P, const LaunchCfg& c)
     return same ? d : c;
 }
 
-LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
-                           uint64_t max_item)
+// Warps per CTA and CTAs per SM of the automatic shape, for mtgp_fast_kernel.
+static LaunchCfg auto_shape(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
+                            uint64_t max_item)
 {
     LaunchCfg c = cfg;
-    if (!cfg.automatic || n_items == 0)
-        return c;
     c.warps_per_cta = 8;
     c.ctas_per_sm = 1;
     const uint64_t sms = (uint64_t)st->sms;
@@ -758,6 +757,20 @@ LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_
         c.warps_per_cta = 4;
         c.ctas_per_sm = 2;
     }
+    return c;
+}
+
+LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
+                           uint64_t max_item)
+{
+    LaunchCfg c = cfg;
+    c.brief = cfg.kernel == 0 && cfg.coop_percent == 0 && brief_items(st->P.k.n, st->sms, n_items, total, max_item);
+    if (!cfg.automatic || n_items == 0)
+        return c;
+    if (!c.brief)
+        return auto_shape(st, c, n_items, total, max_item);
+    c.warps_per_cta = 8;   // 24 warps: all that its registers leave room for
+    c.ctas_per_sm = 3;
     return c;
 }
 
@@ -820,11 +833,12 @@ extern "C" mtgp_status mtgp_get_statuses(mtgp_streams_t st, uint32_t* states, vo
 // memory: the calls that must not enter the allocator come here too).
 mtgp_status mtgp::geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, Geometry* g)
 {
-    const auto key = std::make_tuple(cfg.warps_per_cta, cfg.ctas_per_sm, cfg.k, cfg.kernel);
+    const auto key = std::make_tuple(cfg.warps_per_cta, cfg.ctas_per_sm, cfg.k, cfg.kernel, cfg.brief);
     int at = -1;
     if (cfg.automatic) {
         for (int i = 0; i < kNumAutoShapes; ++i)
-            if (kAutoShapes[i].warps_per_cta == cfg.warps_per_cta && kAutoShapes[i].ctas_per_sm == cfg.ctas_per_sm)
+            if (kAutoShapes[i].warps_per_cta == cfg.warps_per_cta && kAutoShapes[i].ctas_per_sm == cfg.ctas_per_sm &&
+                kAutoShapes[i].brief == cfg.brief)
                 at = i;
     } else {
         for (int i = kNumAutoShapes; i < (int)st->geos.size(); ++i)
@@ -867,6 +881,7 @@ void mtgp::resolve_shapes(mtgp_streams* st)
         LaunchCfg c = st->cfg;
         c.warps_per_cta = sh.warps_per_cta;
         c.ctas_per_sm = sh.ctas_per_sm;
+        c.brief = sh.brief;
         geometry_for(st, c, 1, &g);   // one that cannot launch is reported when a call chooses it
     }
     st->shapes_resolved = true;
@@ -1686,8 +1701,10 @@ static mtgp_status stats_geometry(mtgp_plan* p)
     // an automatic shape of 12 warps (no stream longer than a warp's share
     // there) rounds up: the statistics' latency takes 16 warps to hide
     // (2432 x 2^19, Mexp 23209: 1.94 ms on 16 warps per SM, 2.80 on 8)
-    const int warps = p->cfg.warps_per_cta * p->cfg.ctas_per_sm + (p->cfg.automatic ? G - 1 : 0);
-    if (p->cfg.ctas_per_sm > 0)
+    const LaunchCfg c = p->cfg.automatic && p->n_items
+                            ? auto_shape(st, p->cfg, p->n_items, p->split.work.total, p->max_item) : p->cfg;
+    const int warps = c.warps_per_cta * c.ctas_per_sm + (c.automatic ? G - 1 : 0);
+    if (c.ctas_per_sm > 0)
         per_sm = std::min(per_sm, std::max(1, warps / G));
     cudaFuncAttributes fa;
     CUDA_TRY(cudaFuncGetAttributes(&fa, fn), "cudaFuncGetAttributes");

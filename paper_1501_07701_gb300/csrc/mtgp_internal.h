@@ -66,17 +66,20 @@ struct LaunchCfg {
     int coop_percent;    // streams longer than coop_percent/100 x (numbers per warp
                          // slot) are advanced by a whole CTA; 0 = never
     bool automatic;      // the default: fit_config chooses warps for each launch's work
+    bool brief = false;  // the launch runs mtgp_brief_kernel (set by fit_config, see brief_items)
 };
 
 // Per-warp shared-memory footprint (32-bit words).
 //   fast: S[0 .. N + mirror) rounded up to 4 words (16-byte aligned rows for
 //         the cp.async stage-in).
+//   brief: S[0 .. N), the repeated column 0 and a step's lanes past column N-1.
 //   ring: the warp's REC/TMP tables (32 words), then S[0 .. N) rounded up
 //         to 4 words.
 __host__ __device__ inline uint32_t fast_smem_words(uint32_t n, uint32_t mirror)
 {
     return (n + mirror + 3u) & ~3u;
 }
+__host__ __device__ inline uint32_t brief_smem_words(uint32_t n) { return (n + 129u + 3u) & ~3u; }
 __host__ __device__ inline uint32_t ring_smem_words(uint32_t n) { return 32u + ((n + 3u) & ~3u); }
 
 // True if the register-resident kernel has an instantiation for this N, k
@@ -165,6 +168,7 @@ struct Geometry {
     int regs;            // registers per thread of the kernel used
     int per_sm;          // resident CTAs per SM (occupancy, after the cap)
     int sms;             // SMs of the device
+    const void* fn;      // register-resident and brief kernels: the instantiation
 };
 
 // Works out kernel choice, block size, shared memory and grid (persistent:
@@ -176,14 +180,13 @@ cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_ite
 // Launches the generation kernel described by `g` (counter must be zero).
 cudaError_t launch_generate(const GenArgs& a, const Geometry& g, cudaStream_t s);
 
-// Fast-kernel launchers, one translation unit per group of state sizes.
-// M = ceil(N / 32) register columns per lane; returns cudaErrorInvalidValue
-// if M or K has no instantiation.
-cudaError_t launch_fast(int M, int K, int G, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
-                        uint32_t sms, cudaStream_t s);
+// Instantiations of the register-resident kernel, one translation unit per
+// group of state sizes (M = ceil(N / 32) register columns per lane), and of
+// mtgp_brief_kernel (K sub-steps per step); null where there is none.
 const void* fast_kernel_ptr(int M, int K, int G);
+const void* brief_kernel_ptr(int K, int G);
 
-// Launches a generation kernel with the register-resident kernel's signature.
+// Launches a generation kernel with the register-resident kernel's arguments.
 cudaError_t launch_gen_fn(const void* fn, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
                           uint32_t sms, cudaStream_t s);
 

@@ -267,7 +267,10 @@ cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_ite
     g->k = k;
     g->threads = warps * 32;
     const void* fn;
-    if (kernel == 0) {
+    if (kernel == 0 && cfg.brief) {
+        g->smem = (size_t)warps * brief_smem_words(P.n) * 4u;
+        fn = brief_kernel_ptr(P.n - P.pos >= 128u ? 4 : 2, warps);
+    } else if (kernel == 0) {
         g->smem = (size_t)warps * fast_smem_words(P.n, P.mirror) * 4u;
         fn = fast_kernel_ptr(fast_m(P), k, warps);
     } else {
@@ -289,6 +292,7 @@ cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_ite
     e = cudaFuncGetAttributes(&fa, fn);
     if (e != cudaSuccess)
         return e;
+    g->fn = fn;
     g->regs = fa.numRegs;
     g->per_sm = per_sm;
     int sms = 0;
@@ -307,8 +311,7 @@ cudaError_t launch_generate(const GenArgs& a, const Geometry& g, cudaStream_t s)
     if (a.n_items == 0)
         return cudaSuccess;
     if (g.kernel == 0)
-        return launch_fast((int)((a.P.n + 31u) / 32u), g.k, g.threads / 32, a, dim3(g.grid),
-                           dim3(g.threads), g.smem, (uint32_t)g.sms, s);
+        return launch_gen_fn(g.fn, a, dim3(g.grid), dim3(g.threads), g.smem, (uint32_t)g.sms, s);
     mtgp_ring_kernel<<<g.grid, g.threads, g.smem, s>>>(a.P, a.states, a.n_streams, a.items, a.segs,
                                                        a.n_items, a.counter, a.out, a.err, a.sets,
                                                        a.set_of);
@@ -334,15 +337,6 @@ const void* fast_kernel_ptr(int M, int K, int G)
     if (!p)
         p = fast_ptr_group_d(M, K, G);
     return p;
-}
-
-cudaError_t launch_fast(int M, int K, int G, const GenArgs& a, dim3 grid, dim3 block, size_t smem,
-                        uint32_t sms, cudaStream_t s)
-{
-    const void* fn = fast_kernel_ptr(M, K, G);
-    if (!fn)
-        return cudaErrorInvalidValue;
-    return launch_gen_fn(fn, a, grid, block, smem, sms, s);
 }
 
 cudaError_t launch_gen_fn(const void* fn, const GenArgs& a, dim3 grid, dim3 block, size_t smem,

@@ -41,14 +41,17 @@ struct BuildScratch {
 struct AutoShape {
     int warps_per_cta;
     int ctas_per_sm;
+    bool brief;
 };
-constexpr AutoShape kAutoShapes[] = {{4, 1}, {4, 2}, {4, 3}, {8, 1}, {8, 2}};
+constexpr AutoShape kAutoShapes[] = {{4, 1, false}, {4, 2, false}, {4, 3, false},
+                                     {8, 1, false}, {8, 2, false}, {8, 3, true}};
 constexpr int kNumAutoShapes = (int)(sizeof kAutoShapes / sizeof kAutoShapes[0]);
 
-// Geometry of one configuration (warps per CTA, CTAs per SM, sub-steps, kernel).
+// Geometry of one configuration (warps per CTA, CTAs per SM, sub-steps, kernel,
+// brief).
 struct GeoEntry {
     bool valid = false;
-    std::tuple<int, int, int, int> key{};
+    std::tuple<int, int, int, int, bool> key{};
     Geometry g{};
 };
 
@@ -220,6 +223,20 @@ void fill_table(const Work& w, void* host);
 LaunchCfg default_config(const KParams& P);
 // `c`, or the default configuration if `c` has its values.
 LaunchCfg recognise_default(const KParams& P, const LaunchCfg& c);
+// True if a launch runs mtgp_brief_kernel: more streams than 8 warps per SM
+// (with fewer, each has its place on a warp of mtgp_fast_kernel at once: 1216
+// of 2^2 .. 2^10 at Mexp 44497 in 11.7 us), of at most six rows on average, and
+// of 8 at most or, from 48 streams per SM on, 12.  Measured against
+// mtgp_fast_kernel in the automatic shape, at Mexp 11213 / 23209 / 44497: 10 000
+// equal streams of 5.6 to 5.9 rows 41 and 42 us, 65 and 68, 114 and 135; of 11.3
+// to 11.8 rows 67 and 54, 116 and 90, 200 and 186; uneven ones of up to that
+// many rows 26 and 30, 41 and 46, 68 and 80, but 5000 of them 23 and 21, 36 and
+// 29, 58 and 47.
+inline bool brief_items(uint32_t n, int sms, uint32_t n_items, uint64_t total, uint64_t max_item)
+{
+    const uint64_t rows = n_items >= 48u * (uint32_t)sms ? 12u : 8u;
+    return n_items > 8u * (uint32_t)sms && max_item <= rows * n && total <= 6ull * n * n_items;
+}
 // The configuration a launch of this work runs with: `cfg` itself, or for the
 // default configuration its warps per CTA and CTAs per SM chosen from the
 // number of items, their total and the longest.
