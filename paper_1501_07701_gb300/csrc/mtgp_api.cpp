@@ -760,17 +760,38 @@ static LaunchCfg auto_shape(const mtgp_streams* st, const LaunchCfg& cfg, uint32
     return c;
 }
 
+bool mtgp::general_rows(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
+                        uint64_t max_item)
+{
+    if (st->d_sets || st->P.k.n <= 256u)   // (short states have late loops of their own)
+        return false;
+    const uint32_t sms = (uint32_t)st->sms, warps = cfg.ctas_per_sm ? cfg.warps_per_cta * cfg.ctas_per_sm : 64;
+    const uint32_t fast = st->P.k.n <= 512u && cfg.warps_per_cta <= 4 ? 12 : 8;   // mtgp_fast_kernel's warps
+    if (warps <= fast || max_item * n_items > total + total / 8u)
+        return false;
+    if (cfg.coop_percent == 0)
+        return st->P.k.n - st->P.k.pos < 256u && n_items > 12u * sms;
+    return n_items * (uint32_t)cfg.warps_per_cta > fast * sms &&
+           (uint64_t)n_items * (uint32_t)cfg.coop_percent <= 800ull * sms;
+}
+
 LaunchCfg mtgp::fit_config(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total,
                            uint64_t max_item)
 {
     LaunchCfg c = cfg;
-    c.brief = cfg.kernel == 0 && cfg.coop_percent == 0 && brief_items(st->P.k.n, st->sms, n_items, total, max_item);
-    if (!cfg.automatic || n_items == 0)
+    c.rows = Rows::kLong;
+    if (cfg.kernel == 0 && cfg.coop_percent == 0 && brief_items(st->P.k.n, st->sms, n_items, total, max_item)) {
+        c.rows = Rows::kBrief;
+        if (cfg.automatic) {
+            c.warps_per_cta = 8;   // 24 warps: all that its registers leave room for
+            c.ctas_per_sm = 3;
+        }
         return c;
-    if (!c.brief)
-        return auto_shape(st, c, n_items, total, max_item);
-    c.warps_per_cta = 8;   // 24 warps: all that its registers leave room for
-    c.ctas_per_sm = 3;
+    }
+    if (cfg.automatic && n_items != 0)
+        c = auto_shape(st, c, n_items, total, max_item);
+    if (cfg.kernel == 0 && general_rows(st, c, n_items, total, max_item))
+        c.rows = Rows::kGeneral;
     return c;
 }
 
@@ -833,12 +854,12 @@ extern "C" mtgp_status mtgp_get_statuses(mtgp_streams_t st, uint32_t* states, vo
 // memory: the calls that must not enter the allocator come here too).
 mtgp_status mtgp::geometry_for(mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, Geometry* g)
 {
-    const auto key = std::make_tuple(cfg.warps_per_cta, cfg.ctas_per_sm, cfg.k, cfg.kernel, cfg.brief);
+    const auto key = std::make_tuple(cfg.warps_per_cta, cfg.ctas_per_sm, cfg.k, cfg.kernel, cfg.rows);
     int at = -1;
     if (cfg.automatic) {
         for (int i = 0; i < kNumAutoShapes; ++i)
             if (kAutoShapes[i].warps_per_cta == cfg.warps_per_cta && kAutoShapes[i].ctas_per_sm == cfg.ctas_per_sm &&
-                kAutoShapes[i].brief == cfg.brief)
+                kAutoShapes[i].brief == (cfg.rows == Rows::kBrief))
                 at = i;
     } else {
         for (int i = kNumAutoShapes; i < (int)st->geos.size(); ++i)
@@ -881,7 +902,7 @@ void mtgp::resolve_shapes(mtgp_streams* st)
         LaunchCfg c = st->cfg;
         c.warps_per_cta = sh.warps_per_cta;
         c.ctas_per_sm = sh.ctas_per_sm;
-        c.brief = sh.brief;
+        c.rows = sh.brief ? Rows::kBrief : general_rows(st, c, 1, 1, 1) ? Rows::kGeneral : Rows::kLong;
         geometry_for(st, c, 1, &g);   // one that cannot launch is reported when a call chooses it
     }
     st->shapes_resolved = true;
@@ -952,7 +973,7 @@ mtgp_status mtgp::launch_work_slot(mtgp_streams* st, TableSlot& sl, const Work& 
     // few requests, reads each entry of the table about once, so a small table
     // stays in the pinned host buffer and the warps read it there: no copy for
     // the kernel to wait for.
-    const bool in_place = bytes <= kCounterBytes + kInPlaceTable && g.kernel == 0 && run.coop_percent == 0 &&
+    const bool in_place = bytes <= kCounterBytes + kInPlaceTable && g.places && run.coop_percent == 0 &&
                           items_placed((uint32_t)w.items.size(), (uint32_t)g.grid, (uint32_t)g.threads / 32u) &&
                           std::all_of(w.items.begin(), w.items.end(),
                                       [](const WorkItem& it) { return it.nseg <= kInPlaceRequests; });
@@ -1470,7 +1491,7 @@ static mtgp_status record_graph(mtgp_plan* p)
     a.sets = p->st->d_sets;
     a.set_of = split ? p->d_row_set : p->st->d_set_of;
     a.one_list = one_claim_list(p->max_item);
-    const bool counted = p->stats || p->geo.kernel != 0 || a.n_coop ||
+    const bool counted = p->stats || !p->geo.places || a.n_coop ||
                          !items_placed(p->n_items, (uint32_t)p->geo.grid, (uint32_t)p->geo.threads / 32u);
     if (e1 == cudaSuccess && counted)
         e1 = cudaMemsetAsync(p->d_table, 0, kCounterBytes, cap);

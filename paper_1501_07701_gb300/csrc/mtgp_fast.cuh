@@ -736,15 +736,12 @@ __device__ __forceinline__ void run_single(const KParams& KP, const RowP& P, uin
 {
     if constexpr (M < 9) {   // 32 K <= N - pos, so N - pos >= 64
         run_item_late<M>(KP, P, g, S, segs, s_begin, s_end, out, lane, Tb);
-        return;
-    } else if constexpr (K == 4) {
-        if (P.n - P.pos >= 256u) {
+    } else {
+        if (P.n - P.pos >= 256u)
             run_item_late<M>(KP, P, g, S, segs, s_begin, s_end, out, lane, Tb);
-            return;
-        }
+        else
+            run_item<M, K, 1>(KP, P, g, S, segs, s_begin, s_end, out, warp, lane, Tb);
     }
-    if constexpr (M >= 9)
-        run_item<M, K, 1>(KP, P, g, S, segs, s_begin, s_end, out, warp, lane, Tb);
 }
 
 // Claims.  The n items (longest first) are dealt to n_groups lists, one per
@@ -821,34 +818,30 @@ __device__ __forceinline__ uint32_t claim_item(Claims& c, uint32_t lane)
     }
 }
 
-// Resident CTAs the compiler leaves registers for: 12 warps per SM for the
+// Resident CTAs the compiler leaves registers for in mtgp_fast_kernel: 12 warps per SM for the
 // smaller states (168 registers), 8 for the larger ones, which keep three
 // words per column group.  At 16 warps (128 registers) the late loop spilled
 // and ran at 1190 instead of 1400 Gnumbers/s (2432 equal streams, Mexp 11213).
 // Short states, with a chain of 32-column sub-steps to hide, run best at 16
 // (2432 equal streams at Mexp 3217: 1098 Gnumbers/s; at 24 and 32 warps per SM
-// the loop spills and runs at 840); the other row loops need few registers.
-constexpr int fast_min_ctas(int M, int K, int G)
+// the loop spills and runs at 840).
+constexpr int fast_min_ctas(int M, int G)
 {
-    return (M < 9 || K != 4 ? 16 : M < 16 ? 12 : 8) / G;
+    return (M < 9 ? 16 : M < 16 ? 12 : 8) / G;
 }
 
 // Persistent kernel.  Phase 1: the CTA claims the longest streams (items
 // [0, n_coop) of the table, sorted longest first) one at a time and its G
 // warps advance each together.  Phase 2: every warp claims the remaining
 // items [n_coop, n_items) one by one and advances each alone.
+#define MTGP_KERNEL_PARAMS                                                                       \
+    uint32_t *__restrict__ states, uint32_t n_streams, const WorkItem *__restrict__ items,       \
+        const Segment *__restrict__ segs, uint32_t n_items, uint32_t n_coop,                     \
+        uint32_t *__restrict__ counters, uint32_t *__restrict__ out, int *__restrict__ err,      \
+        uint64_t *__restrict__ trace, const KSet *__restrict__ sets,                             \
+        const uint32_t *__restrict__ set_of, uint32_t n_groups
 template <int M, int K, int G>
-__global__ void __launch_bounds__(G * 32, fast_min_ctas(M, K, G)) mtgp_fast_kernel(const KParams P, uint32_t* __restrict__ states,
-                                                           uint32_t n_streams,
-                                                           const WorkItem* __restrict__ items,
-                                                           const Segment* __restrict__ segs,
-                                                           uint32_t n_items, uint32_t n_coop,
-                                                           uint32_t* __restrict__ counters,
-                                                           uint32_t* __restrict__ out, int* __restrict__ err,
-                                                           uint64_t* __restrict__ trace,
-                                                           const KSet* __restrict__ sets,
-                                                           const uint32_t* __restrict__ set_of,
-                                                           uint32_t n_groups)
+__global__ void __launch_bounds__(G * 32, fast_min_ctas(M, G)) mtgp_fast_kernel(const KParams P, MTGP_KERNEL_PARAMS)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ uint32_t s_claim;
@@ -936,6 +929,86 @@ __global__ void __launch_bounds__(G * 32, fast_min_ctas(M, K, G)) mtgp_fast_kern
         } else {
             run_single<M, K>(P, R0, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
                              w.seg_begin + w.nseg, out, warp, lane, Tb[0]);
+        }
+        if (trace && lane == 0)
+            trace_item(trace, it, t0, segs, w);
+    }
+}
+
+// Without the late-tempering loops: for steps of 256 words (K = 8) and where
+// general_rows chooses it.  Its loops need few registers, so the compiler is
+// left to choose (64 to 128, 16 to 32 warps per SM).  In one kernel with claims
+// by place or from lists per SM the K = 8 loops came out 5 to 18 % slower (8
+// warps per SM, 4096 x 2^16 at Mexp 11213: 334 us, 377 there), so items are
+// claimed from one list, counters[1], always.
+template <int M, int K, int G>
+__global__ void __launch_bounds__(G * 32) mtgp_general_kernel(const KParams P, MTGP_KERNEL_PARAMS)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ uint32_t s_claim;
+    __shared__ __align__(64) uint32_t Tb[G][48];   // 192-byte rows: every table starts on a 64-byte boundary
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t warp = threadIdx.x >> 5;
+    if (threadIdx.x < 16) {
+        Tb[0][threadIdx.x] = P.rec[threadIdx.x];
+        Tb[0][16 + threadIdx.x] = P.tmp[threadIdx.x];
+        Tb[0][32 + threadIdx.x] = P.flt[threadIdx.x];
+    }
+    __syncthreads();
+    const RowP R0 = {P.n, P.mask, P.pos, P.sh1, P.sh2, P.mirror};
+    const uint32_t first_single = (K >= G && !sets) ? n_coop : 0u;
+    if constexpr (K >= G) {
+    for (; !sets;) {
+        if (threadIdx.x == 0)
+            s_claim = atomicAdd(&counters[0], 1u);
+        __syncthreads();
+        const uint32_t it = s_claim;
+        __syncthreads();
+        if (it >= n_coop)
+            break;
+        const WorkItem w = items[it];
+        if (w.stream >= n_streams || w.nseg == 0) {
+            if (threadIdx.x == 0)
+                atomicOr(err, 1);
+            continue;
+        }
+        const uint64_t t0 = trace ? global_ns() : 0;
+        run_item<M, K, G>(P, R0, states + (size_t)w.stream * P.np, smem, segs, w.seg_begin,
+                          w.seg_begin + w.nseg, out, warp, lane, Tb[0]);
+        if (trace && threadIdx.x == 0)
+            trace_item(trace, it, t0, segs, w);
+    }
+    }
+    uint32_t* S = smem + warp * fast_smem_words(P.n, P.mirror);
+    for (;;) {
+        uint32_t it = 0;
+        if (lane == 0)
+            it = first_single + atomicAdd(&counters[1], 1u);
+        it = __shfl_sync(MTGP_FULL, it, 0);
+        if (it >= n_items)
+            break;
+        const WorkItem w = items[it];
+        if (w.stream >= n_streams || w.nseg == 0) {
+            if (lane == 0)
+                atomicOr(err, 1);
+            continue;
+        }
+        const uint64_t t0 = trace ? global_ns() : 0;
+        if (sets) {
+            // this stream's own parameter set
+            const KSet& ks = sets[set_of[w.stream]];
+            const RowP R = {P.n, P.mask, ks.pos, ks.sh1, ks.sh2, ks.mirror};
+            if (lane < 16u) {
+                Tb[warp][lane] = ks.rec[lane];
+                Tb[warp][16u + lane] = ks.tmp[lane];
+                Tb[warp][32u + lane] = ks.flt[lane];
+            }
+            __syncwarp();
+            run_item<M, K, 1>(P, R, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
+                              w.seg_begin + w.nseg, out, warp, lane, Tb[warp]);
+        } else {
+            run_item<M, K, 1>(P, R0, states + (size_t)w.stream * P.np, S, segs, w.seg_begin,
+                              w.seg_begin + w.nseg, out, warp, lane, Tb[0]);
         }
         if (trace && lane == 0)
             trace_item(trace, it, t0, segs, w);

@@ -5,15 +5,15 @@
 
 namespace mtgp {
 
-const void* fast_ptr_group_c(int M, int K, int G)
+const void* fast_ptr_group_c(int M, int K, int G, bool general)
 {
     switch ((M * 16 + K) * 16 + G) {
-    case (44 * 16 + 8) * 16 + 2: return (const void*)mtgp_fast_kernel<44, 8, 2>;
-    case (44 * 16 + 8) * 16 + 4: return (const void*)mtgp_fast_kernel<44, 8, 4>;
-    case (44 * 16 + 8) * 16 + 8: return (const void*)mtgp_fast_kernel<44, 8, 8>;
-    case (44 * 16 + 4) * 16 + 2: return (const void*)mtgp_fast_kernel<44, 4, 2>;
-    case (44 * 16 + 4) * 16 + 4: return (const void*)mtgp_fast_kernel<44, 4, 4>;
-    case (44 * 16 + 4) * 16 + 8: return (const void*)mtgp_fast_kernel<44, 4, 8>;
+    case (44 * 16 + 8) * 16 + 2: return (const void*)mtgp_general_kernel<44, 8, 2>;
+    case (44 * 16 + 8) * 16 + 4: return (const void*)mtgp_general_kernel<44, 8, 4>;
+    case (44 * 16 + 8) * 16 + 8: return (const void*)mtgp_general_kernel<44, 8, 8>;
+    case (44 * 16 + 4) * 16 + 2: return general ? (const void*)mtgp_general_kernel<44, 4, 2> : (const void*)mtgp_fast_kernel<44, 4, 2>;
+    case (44 * 16 + 4) * 16 + 4: return general ? (const void*)mtgp_general_kernel<44, 4, 4> : (const void*)mtgp_fast_kernel<44, 4, 4>;
+    case (44 * 16 + 4) * 16 + 8: return general ? (const void*)mtgp_general_kernel<44, 4, 8> : (const void*)mtgp_fast_kernel<44, 4, 8>;
     default: return nullptr;
     }
 }

@@ -7,7 +7,7 @@
 
 namespace mtgp {
 
-const void* fast_ptr_group_d(int M, int K, int G)
+const void* fast_ptr_group_d(int M, int K, int G, bool)
 {
     switch ((M * 16 + K) * 16 + G) {
     case (4 * 16 + 2) * 16 + 2: return (const void*)mtgp_fast_kernel<4, 2, 2>;

@@ -58,6 +58,13 @@ struct Segment {
     uint32_t req;
 };
 
+// The kernels of the register-resident path.
+enum class Rows {
+    kLong,      // mtgp_fast_kernel
+    kBrief,     // mtgp_brief_kernel: many short streams (brief_items)
+    kGeneral,   // mtgp_general_kernel (general_rows)
+};
+
 struct LaunchCfg {
     int warps_per_cta;   // G: 2, 4 or 8 for the register-resident kernel (1..8 ring)
     int ctas_per_sm;     // 0 = occupancy maximum
@@ -66,7 +73,7 @@ struct LaunchCfg {
     int coop_percent;    // streams longer than coop_percent/100 x (numbers per warp
                          // slot) are advanced by a whole CTA; 0 = never
     bool automatic;      // the default: fit_config chooses warps for each launch's work
-    bool brief = false;  // the launch runs mtgp_brief_kernel (set by fit_config, see brief_items)
+    Rows rows = Rows::kLong;   // kernel 0: which of its kernels (set by fit_config)
 };
 
 // Per-warp shared-memory footprint (32-bit words).
@@ -168,7 +175,8 @@ struct Geometry {
     int regs;            // registers per thread of the kernel used
     int per_sm;          // resident CTAs per SM (occupancy, after the cap)
     int sms;             // SMs of the device
-    const void* fn;      // register-resident and brief kernels: the instantiation
+    const void* fn;      // register-resident path: the kernel's instantiation
+    bool places;         // it gives items to warps by their place where it can (items_placed)
 };
 
 // Works out kernel choice, block size, shared memory and grid (persistent:
@@ -183,7 +191,7 @@ cudaError_t launch_generate(const GenArgs& a, const Geometry& g, cudaStream_t s)
 // Instantiations of the register-resident kernel, one translation unit per
 // group of state sizes (M = ceil(N / 32) register columns per lane), and of
 // mtgp_brief_kernel (K sub-steps per step); null where there is none.
-const void* fast_kernel_ptr(int M, int K, int G);
+const void* fast_kernel_ptr(int M, int K, int G, bool general);
 const void* brief_kernel_ptr(int K, int G);
 
 // Launches a generation kernel with the register-resident kernel's arguments.

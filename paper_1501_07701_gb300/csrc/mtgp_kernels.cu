@@ -239,7 +239,7 @@ bool fast_supported(const KParams& P, int k, int g)
     const int M = fast_m(P);
     if (M <= k)
         return false;
-    return fast_kernel_ptr(M, k, g) != nullptr;
+    return fast_kernel_ptr(M, k, g, false) != nullptr;
 }
 
 cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_items, int device,
@@ -267,12 +267,12 @@ cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_ite
     g->k = k;
     g->threads = warps * 32;
     const void* fn;
-    if (kernel == 0 && cfg.brief) {
+    if (kernel == 0 && cfg.rows == Rows::kBrief) {
         g->smem = (size_t)warps * brief_smem_words(P.n) * 4u;
         fn = brief_kernel_ptr(P.n - P.pos >= 128u ? 4 : 2, warps);
     } else if (kernel == 0) {
         g->smem = (size_t)warps * fast_smem_words(P.n, P.mirror) * 4u;
-        fn = fast_kernel_ptr(fast_m(P), k, warps);
+        fn = fast_kernel_ptr(fast_m(P), k, warps, cfg.rows == Rows::kGeneral);
     } else {
         g->smem = (size_t)warps * ring_smem_words(P.n) * 4u;
         fn = (const void*)mtgp_ring_kernel;
@@ -293,6 +293,7 @@ cudaError_t plan_geometry(const KParams& P, const LaunchCfg& cfg, uint32_t n_ite
     if (e != cudaSuccess)
         return e;
     g->fn = fn;
+    g->places = kernel == 0 && (cfg.rows == Rows::kBrief || fast_m(P) < 9 || (k == 4 && cfg.rows == Rows::kLong));
     g->regs = fa.numRegs;
     g->per_sm = per_sm;
     int sms = 0;
@@ -322,20 +323,20 @@ cudaError_t launch_generate(const GenArgs& a, const Geometry& g, cudaStream_t s)
 
 namespace mtgp {
 
-const void* fast_ptr_group_a(int M, int K, int G);
-const void* fast_ptr_group_b(int M, int K, int G);
-const void* fast_ptr_group_c(int M, int K, int G);
-const void* fast_ptr_group_d(int M, int K, int G);
+const void* fast_ptr_group_a(int M, int K, int G, bool general);
+const void* fast_ptr_group_b(int M, int K, int G, bool general);
+const void* fast_ptr_group_c(int M, int K, int G, bool general);
+const void* fast_ptr_group_d(int M, int K, int G, bool general);
 
-const void* fast_kernel_ptr(int M, int K, int G)
+const void* fast_kernel_ptr(int M, int K, int G, bool general)
 {
-    const void* p = fast_ptr_group_a(M, K, G);
+    const void* p = fast_ptr_group_a(M, K, G, general);
     if (!p)
-        p = fast_ptr_group_b(M, K, G);
+        p = fast_ptr_group_b(M, K, G, general);
     if (!p)
-        p = fast_ptr_group_c(M, K, G);
+        p = fast_ptr_group_c(M, K, G, general);
     if (!p)
-        p = fast_ptr_group_d(M, K, G);
+        p = fast_ptr_group_d(M, K, G, general);
     return p;
 }
 

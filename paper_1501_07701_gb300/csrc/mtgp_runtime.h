@@ -48,10 +48,10 @@ constexpr AutoShape kAutoShapes[] = {{4, 1, false}, {4, 2, false}, {4, 3, false}
 constexpr int kNumAutoShapes = (int)(sizeof kAutoShapes / sizeof kAutoShapes[0]);
 
 // Geometry of one configuration (warps per CTA, CTAs per SM, sub-steps, kernel,
-// brief).
+// its rows).
 struct GeoEntry {
     bool valid = false;
-    std::tuple<int, int, int, int, bool> key{};
+    std::tuple<int, int, int, int, Rows> key{};
     Geometry g{};
 };
 
@@ -237,6 +237,15 @@ inline bool brief_items(uint32_t n, int sms, uint32_t n_items, uint64_t total, u
     const uint64_t rows = n_items >= 48u * (uint32_t)sms ? 12u : 8u;
     return n_items > 8u * (uint32_t)sms && max_item <= rows * n && total <= 6ull * n * n_items;
 }
+// True if a launch that is not brief runs mtgp_general_kernel (which is also
+// the only kernel for words_per_lane 8): its configuration asks for more warps
+// than mtgp_fast_kernel's 8 or 12 per SM, its streams are about equal, and none
+// would take the late-tempering loops.  Either a CTA-wide phase takes all of
+// them (no more than 8 per SM, and more than mtgp_fast_kernel has CTAs for: 1216
+// of 2^16 with coop_percent 100 at Mexp 11213 153 us, 301 there), or there are many and the parameter set has N - pos < 256
+// (4096 of 2^16 at Mexp 23209 in 20 warps per SM 268 us, 346 there; uneven ones
+// lose more by such residency than they gain, 1.3 against 0.92 ms).
+bool general_rows(const mtgp_streams* st, const LaunchCfg& cfg, uint32_t n_items, uint64_t total, uint64_t max_item);
 // The configuration a launch of this work runs with: `cfg` itself, or for the
 // default configuration its warps per CTA and CTAs per SM chosen from the
 // number of items, their total and the longest.
