@@ -112,7 +112,7 @@ __device__ __forceinline__ void mt_sts(uint32_t a, uint32_t v)
 // What bounds it: that chain, 130 cycles per step for a warp alone and 172 for
 // two warps per SM quarter (p = 3217, 51 numbers per step).  Measured, uneven
 // 10 000-stream workload, against the loop that loaded all three words first
-// and tempered the previous step after: p = 3217 7.70 -> 6.97 ms, MT19937 7.16
+// and tempered the previous step after: p = 3217 7.74 -> 6.52 ms, MT19937 7.16
 // -> 5.93, p = 44497 7.32 -> 6.33.  Reading a whole step ahead, with the one or
 // two words it then lacks at p = 3217 by shuffle, took more instructions than
 // it hid latency (9.6 ms).

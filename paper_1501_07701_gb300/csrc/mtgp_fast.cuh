@@ -269,12 +269,12 @@ __device__ __forceinline__ void gen_row(uint32_t (&r)[(M + WG - 1) / WG], uint32
 // row they are simply unused.  Before the first row these loads are made apart,
 // and the numbers after the loop read neighbours' words too, which a run that
 // follows at once (a request that ends with a row) overwrites in its step 0: a
-// barrier before the loop orders both before step 0's stores.  Lanes past column N-1 in the last group
-// compute on the words behind the row and write there; only their output
-// store is predicated off.
+// barrier before the loop orders both before step 0's stores.  Lanes past
+// column N-1 in the last group compute on the words behind the row and write
+// there; only their output store is predicated off.
 //
 // What bounds it (ncu, 1216 streams, 8 warps per SM, Mexp 11213): 6.03 LSU and
-// 11.4 ALU instructions per 32 numbers, LSU data stage 85 % and ALU 74 % busy
+// 10.0 ALU instructions per 32 numbers, LSU data stage 91 % and ALU 70 % busy
 // (the loop it replaced: 7.34 and 13.3).  Hence the late tempering and the
 // wrapped addresses (LSU), the packed folds and the multiply for the left
 // shift (ALU).  Only the packed tempering indices are kept for a row, a
@@ -355,6 +355,16 @@ __device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const R
     // see through: the FMA pipe is idle, the ALU pipe is not
     uint32_t mul1 = 1u << P.sh1;
     asm volatile("" : "+r"(mul1), "+r"(sa), "+r"(x1_last), "+r"(tb));
+    const uint32_t t0 = temper_index(S[P.pos - 1u]);
+    uint32_t x1[K], xp[K];
+    static_assert(M >= K, "step 0 fills all of x1 and xp");
+    static_for<K>([&](auto ii) {
+        constexpr int i = ii.value;
+        const uint32_t p = 32u * i + lane + P.pos;
+        x1[i] = lds_at<128 * i + 4>(sa);
+        xp[i] = lds_at<0>(saddr(S + (p < N ? p : p - N)));
+    });
+    __syncwarp();   // these loads, and the last ones of a run before, come before step 0's stores
     uint32_t r[M], qa[M];
     uint32_t T[NS];   // the steps' tempering indices, packed
     static_for<M>([&](auto im) {
@@ -365,15 +375,7 @@ __device__ __forceinline__ void gen_rows_late(uint32_t* S, uint32_t* ow, const R
         asm volatile("" : "+r"(qa[m]));   // kept, not worked out again in the loop
     });
     static_for<NS>([&](auto is) { T[is.value] = 0u; });
-    T[NS - 1] = (temper_index(S[P.pos - 1u]) & 15u) << (2 + 8 * ((M - 1) & 3));
-    uint32_t x1[K], xp[K];
-    static_assert(M >= K, "step 0 fills all of x1 and xp");
-    static_for<K>([&](auto ii) {
-        constexpr int i = ii.value;
-        x1[i] = lds_at<128 * i + 4>(sa);
-        xp[i] = lds_at<0>(qa[i]);
-    });
-    __syncwarp();   // these loads, and the last ones of a run before, come before step 0's stores
+    T[NS - 1] = (t0 & 15u) << (2 + 8 * ((M - 1) & 3));
     uint32_t* op = ow + 1 - (int)N;   // where column `lane` of this row stores
 #pragma unroll U
     for (uint32_t q = 0; q < nfull; ++q, op += N) {
@@ -461,6 +463,11 @@ __device__ __forceinline__ void gen_rows_short(uint32_t* S, uint32_t* ow, const 
     uint32_t tb = saddr(Tb);
     uint32_t mul1 = 1u << P.sh1;   // on the FMA pipe, as in gen_rows_late
     asm volatile("" : "+r"(mul1), "+r"(sa), "+r"(x1_last), "+r"(tb));
+    // what other lanes write is read before the barrier (as in gen_rows_late);
+    // the loop is 1.5 % faster for these loads standing first
+    const uint32_t p0 = lane + P.pos, t0 = temper_index(S[P.pos - 1u]);
+    uint32_t x1 = lds_at<4>(sa), xp = lds_at<0>(saddr(S + (p0 < N ? p0 : p0 - N)));
+    __syncwarp();
     uint32_t r[M], qa[M], T[NT], xs[4 * NT];
     static_for<M>([&](auto im) {
         constexpr int m = im.value;
@@ -471,9 +478,7 @@ __device__ __forceinline__ void gen_rows_short(uint32_t* S, uint32_t* ow, const 
     });
     static_for<NT>([&](auto i) { T[i.value] = 0u; });
     static_for<4 * NT>([&](auto i) { xs[i.value] = 0u; });
-    T[NT - 1] = (temper_index(S[P.pos - 1u]) & 15u) << (2 + 8 * ((M - 1) & 3));
-    uint32_t x1 = lds_at<4>(sa), xp = lds_at<0>(qa[0]);
-    __syncwarp();   // as in gen_rows_late
+    T[NT - 1] = (t0 & 15u) << (2 + 8 * ((M - 1) & 3));
     uint32_t* op = ow + 1 - (int)N;
 #pragma unroll 4
     for (uint32_t q = 0; q < nfull; ++q, op += N) {
@@ -847,8 +852,8 @@ __global__ void __launch_bounds__(G * 32, fast_min_ctas(M, G)) mtgp_fast_kernel(
     __shared__ uint32_t s_claim;
     // Tables: Tb[0] holds the handle's set; with per-stream sets each warp
     // loads its stream's tables into its own Tb[warp] (256-byte rows: every
-    // table is 64-byte aligned, entry k in bank k, and temper_addr needs the
-    // row's address to end in a zero byte).
+    // table is 64-byte aligned, entry k in bank k, and the address of a row ends
+    // in a zero byte, under which the late loops put a packed tempering index).
     __shared__ __align__(256) uint32_t Tb[G][64];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = threadIdx.x >> 5;

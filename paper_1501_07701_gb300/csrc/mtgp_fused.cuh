@@ -324,7 +324,7 @@ __device__ __forceinline__ void ham_step(const uint32_t (&w)[4], uint32_t step_n
 // of the loop.  Measured (one launch, 5.12 G numbers, Mexp 11213): 14.0 -> 10.6
 // ms at 8 warps per SM, 10.3 -> 7.35 ms at 16 split in pieces of 1 052 897;
 // 2432 x 2^19 at Mexp 23209 and 16 warps per SM 2.44 -> 1.94 ms, at Mexp 44497
-// 2.55 -> 2.24 ms.  What bounds it: issue and latency, about 165 instructions
+// 2.55 -> 2.24 ms.  What bounds it: issue and latency, about 168 instructions
 // per 128 numbers.
 template <int M, int FMT, bool STEPH>
 __device__ __forceinline__ void fused_rows(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,

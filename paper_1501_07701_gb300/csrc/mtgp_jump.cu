@@ -1034,7 +1034,7 @@ cudaError_t mtgp::launch_jump_batch(const mtgp_streams* st, const uint32_t* from
     // jumps 53 -> 51 and 92 -> 86 us against one CTA per SM, 152 jumps 66 ->
     // 62 and 142 -> 118; four per SM is slower again (81 and 152).
     // 10 000 jumps at Mexp 11213 take 1.21 ms, 18 SM-us each (56 before the
-    // sliding windows): 117 000 warp instructions, issue 76 % busy.
+    // sliding windows): 117 000 warp instructions, issue 75 % busy.
     uint32_t parts = 1;
     while (parts < 8u && parts * n <= (uint32_t)st->sms)
         parts *= 2u;
