@@ -731,7 +731,11 @@ static LaunchCfg auto_shape(const mtgp_streams* st, const LaunchCfg& cfg, uint32
     c.warps_per_cta = 8;
     c.ctas_per_sm = 1;
     const uint64_t sms = (uint64_t)st->sms;
-    if (n_items <= 4u * sms) {
+    if (n_items <= sms && st->P.k.n > 256u && st->P.k.n <= 1024u) {
+        // one busy warp per SM: the 8-warp instantiation, which has the most
+        // registers, runs a lone stream fastest (2^20 numbers at Mexp 11213:
+        // 0.515 ms, 0.566 on 4-warp CTAs; 23209: 0.541 and 0.550)
+    } else if (n_items <= 4u * sms) {
         // one warp per SM quarter: a second one on the same quarter slows
         // both (456 streams of 2^20, Mexp 11213: 0.93 ms on 8-warp CTAs
         // whose three busy warps may share a quarter, 0.53 apart)
