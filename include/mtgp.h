@@ -229,9 +229,15 @@ mtgp_status mtgp_streams_free(mtgp_streams_t streams);
 typedef struct {
     uint32_t warps_per_cta;   /* block size / 32: 1..8 (the register-resident
                                  path uses 2, 4 or 8)                          */
-    uint32_t ctas_per_sm;     /* resident CTAs per SM (0 = occupancy maximum)   */
+    uint32_t ctas_per_sm;     /* resident CTAs per SM (0 = occupancy maximum);
+                                 fewer where the registers or shared memory of
+                                 the kernel for the state size leave no room:
+                                 8 to 12 warps per SM for the 128-word steps of
+                                 long streams (mtgp_plan_get_info reports it)  */
     uint32_t words_per_lane;  /* sub-steps per parallel step (2, 4 or 8); the
-                                 window is 32 * words_per_lane <= N - pos      */
+                                 window is 32 * words_per_lane <= N - pos
+                                 (launches of many short streams choose their
+                                 own step)                                     */
     uint32_t kernel;          /* 0 = register-resident path when available,
                                  1 = shared-memory ring path (any parameters)  */
     uint32_t coop_percent;    /* streams of a launch longer than coop_percent/100
