@@ -1705,7 +1705,7 @@ static mtgp_status stats_geometry(mtgp_plan* p)
     const KParams& P = st->P.k;
     const int G = 8;
     const int M = (int)((P.n + 31u) / 32u);
-    const void* fn = fused_kernel_ptr(M, G);
+    const void* fn = fused_kernel_ptr(M, G, p->sa.gmask);
     if (!fn)
         return fail(MTGP_EINVAL, "statistics: no fused kernel for N = %u (ceil(N/32) = %d)", P.n, M);
     // 128-word pipelined rows need N - pos >= 256; short states (M < 9) run

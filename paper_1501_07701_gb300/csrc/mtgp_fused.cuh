@@ -326,7 +326,13 @@ __device__ __forceinline__ void ham_step(const uint32_t (&w)[4], uint32_t step_n
 // 2432 x 2^19 at Mexp 23209 and 16 warps per SM 2.44 -> 1.94 ms, at Mexp 44497
 // 2.55 -> 2.24 ms.  What bounds it: issue and latency, about 168 instructions
 // per 128 numbers.
-template <int M, int FMT, bool STEPH>
+//
+// DENSE: the visits of every sub-step are resolved as they come instead.  A
+// window takes as many passes as its fullest word has visits, so where one
+// value in four or two visits it is slower: 1216 x 2^16 with b = 1 at Mexp 11213
+// 289 us by windows and 232 by sub-steps, at 44497 411 and 238, there also with
+// b = 3 282 and 237 (with b = 5, by windows, 186 and 235).
+template <int M, int FMT, bool STEPH, bool DENSE = false>
 __device__ __forceinline__ void fused_rows(uint32_t* S, uint32_t* ow, const RowP& P, uint32_t lane,
                                            const uint32_t* __restrict__ Tb, uint32_t nfull, StatsState& st,
                                            uint32_t* h, uint32_t* tab, const StatsArgs& A)
@@ -407,23 +413,27 @@ __device__ __forceinline__ void fused_rows(uint32_t* S, uint32_t* ow, const RowP
                     const bool valid = m + 1 < M || lane <= last_lane;
                     if (valid)
                         __stcs(op + 32 * m, o[i]);
-                    const uint32_t B = __ballot_sync(MTGP_FULL, valid && (o[i] & A.gmask) == 0u);
-                    vw = slot == (uint32_t)(M <= 32 ? m : m & 31) ? B : vw;
+                    if constexpr (DENSE) {
+                        count_at(gap_run(o[i], valid, 0u, m + 1 < M ? 32u : nlast, lane, lower, st, hs, own, A));
+                    } else {
+                        const uint32_t B = __ballot_sync(MTGP_FULL, valid && (o[i] & A.gmask) == 0u);
+                        vw = slot == (uint32_t)(M <= 32 ? m : m & 31) ? B : vw;
+                    }
                     w[i] = valid ? __popc(o[i] & A.hmask) : 0u;
                     if constexpr (!STEPH)
                         ham_run(w[i], 0u, m + 1 < M ? 32u : nlast, lane, st, tab, A);
                 });
                 if constexpr (STEPH)
                     ham_step<KS>(w, lasts ? 32u * (KS - 1) + nlast : 32u * KS, lane, st, tab, A);
-                if constexpr (M > 32 && s0 + KS == 32) {
+                if constexpr (!DENSE && M > 32 && s0 + KS == 32) {
                     gap_window(vw, base, 1024u, lane, lower, st, hs, own, A);
                     vw = 0u;
                 }
-                if constexpr (lasts && M > 32) {
+                if constexpr (!DENSE && lasts && M > 32) {
                     gap_window(vw, base, N - 1024u, lane, lower, st, hs, own, A);
                     vw = 0u;
                 }
-                if constexpr (lasts && M <= 32) {
+                if constexpr (!DENSE && lasts && M <= 32) {
                     slot -= (uint32_t)M;
                     if (++rb == (uint32_t)RB) {
                         gap_window(vw, base, RB * N, lane, lower, st, hs, own, A);
@@ -590,7 +600,7 @@ __device__ __forceinline__ void fused_row_slow(uint32_t* S, const RowP& P, uint3
 
 // Advances one stream (this warp alone) by the segments [s_begin, s_end),
 // with the statistics of every request.
-template <int M>
+template <int M, bool DENSE>
 __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uint32_t* __restrict__ g,
                                            uint32_t* S, const Segment* __restrict__ segs, uint32_t s_begin,
                                            uint32_t s_end, uint32_t* __restrict__ out, uint32_t lane,
@@ -634,18 +644,18 @@ __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uin
                     fused_rows_short<M, 2>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
             } else if (A.K >= 128u) {
                 if (sg.fmt == 0)
-                    fused_rows<M, 0, true>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
+                    fused_rows<M, 0, true, DENSE>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else if (sg.fmt == 1)
-                    fused_rows<M, 1, true>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
+                    fused_rows<M, 1, true, DENSE>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else
-                    fused_rows<M, 2, true>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
+                    fused_rows<M, 2, true, DENSE>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
             } else {
                 if (sg.fmt == 0)
-                    fused_rows<M, 0, false>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
+                    fused_rows<M, 0, false, DENSE>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else if (sg.fmt == 1)
-                    fused_rows<M, 1, false>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
+                    fused_rows<M, 1, false, DENSE>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
                 else
-                    fused_rows<M, 2, false>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
+                    fused_rows<M, 2, false, DENSE>(S, ow, P, lane, Tb, nfull, st, h, tab, A);
             }
             row += (uint64_t)nfull * N;
         } else {
@@ -669,8 +679,8 @@ __device__ __forceinline__ void fused_item(const KParams& KP, const RowP& P, uin
 // registers, for 16 warps per SM, also where that spills (M = 44: 450 loads in
 // the whole kernel): 2432 x 2^19 at Mexp 44497 takes 2.24 ms at 16 warps, and
 // 2.53 at the 8 that its 255 registers would leave room for.
-template <int M, int G>
-__global__ void __launch_bounds__(G * 32, 2) mtgp_fused_kernel(const KParams P, uint32_t* __restrict__ states,
+template <int M, int G, bool DENSE = false>
+__global__ void __launch_bounds__(G * 32, DENSE && M > 32 ? 1 : 2) mtgp_fused_kernel(const KParams P, uint32_t* __restrict__ states,
                                                             uint32_t n_streams,
                                                             const WorkItem* __restrict__ items,
                                                             const Segment* __restrict__ segs,
@@ -725,10 +735,10 @@ __global__ void __launch_bounds__(G * 32, 2) mtgp_fused_kernel(const KParams P, 
                 Tb[warp][32u + lane] = ks.flt[lane];
             }
             __syncwarp();
-            fused_item<M>(P, R, g, S, segs, w.seg_begin, w.seg_begin + w.nseg, out, lane, Tb[warp], st,
+            fused_item<M, DENSE>(P, R, g, S, segs, w.seg_begin, w.seg_begin + w.nseg, out, lane, Tb[warp], st,
                           h, tab, A);
         } else {
-            fused_item<M>(P, R0, g, S, segs, w.seg_begin, w.seg_begin + w.nseg, out, lane, Tb[0], st, h,
+            fused_item<M, DENSE>(P, R0, g, S, segs, w.seg_begin, w.seg_begin + w.nseg, out, lane, Tb[0], st, h,
                           tab, A);
         }
     }

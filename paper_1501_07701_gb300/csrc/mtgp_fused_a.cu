@@ -7,6 +7,9 @@ namespace mtgp {
 
 const void* fused_ptr_group_b(int M, int G);
 const void* fused_ptr_group_c(int M, int G);
+const void* fused_ptr_group_d(int M, int G);
+const void* fused_ptr_group_e(int M, int G);
+const void* fused_ptr_group_f(int M, int G);
 
 static const void* fused_ptr_group_a(int M, int G)
 {
@@ -18,9 +21,14 @@ static const void* fused_ptr_group_a(int M, int G)
     }
 }
 
-const void* fused_kernel_ptr(int M, int G)
+const void* fused_kernel_ptr(int M, int G, uint32_t gmask)
 {
-    const void* p = fused_ptr_group_a(M, G);
+    const int b = __builtin_popcount(gmask);   // one value in 2^b visits
+    const void* p = nullptr;
+    if (b <= (M > 32 ? 3 : 2) && !(p = fused_ptr_group_d(M, G)) && !(p = fused_ptr_group_e(M, G)))
+        p = fused_ptr_group_f(M, G);           // (short states have one form)
+    if (!p)
+        p = fused_ptr_group_a(M, G);
     if (!p)
         p = fused_ptr_group_b(M, G);
     return p ? p : fused_ptr_group_c(M, G);

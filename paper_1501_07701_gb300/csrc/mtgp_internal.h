@@ -239,10 +239,10 @@ __host__ __device__ inline uint32_t stats_smem_words(uint32_t t, uint32_t C)
 }
 
 // The fused generation kernel (single-warp items, 128-word pipelined steps,
-// N - pos >= 256 for every parameter set): null when M or G has no
-// instantiation.  Launched like the register-resident kernel plus `A`
+// N - pos >= 256 for every parameter set) for a gap test with this mask: null
+// when M or G has no instantiation.  Launched like the register-resident kernel plus `A`
 // (a.n_coop and a.trace are not used).
-const void* fused_kernel_ptr(int M, int G);
+const void* fused_kernel_ptr(int M, int G, uint32_t gmask);
 cudaError_t launch_fused(const void* fn, const GenArgs& a, const StatsArgs& A, dim3 grid, dim3 block,
                          size_t smem, cudaStream_t s);
 // Completes the statistics of split requests from their pieces' records:
